@@ -7,7 +7,7 @@
 // tcgen05 GEMM, persistent, one CTA per SM, 192 threads:
 //   warp 0, one thread  TMA producer: per k-block a 128 x 64 tile of H and a
 //                       256 x 64 tile of W (128-byte swizzle) into a 4-stage ring
-//   warp 1, one thread  MMA issuer (M128 N256 K16, bf16 -> f32) into one of two
+//   warp 1, converged   MMA issuer (M128 N256 K16, bf16 -> f32) into one of two
 //                       TMEM accumulators of 256 columns; allocates TMEM
 //   warps 2-5           epilogue: each thread owns one row of the 128 x 256
 //                       accumulator, reads it from TMEM 32 columns at a time,
@@ -131,9 +131,14 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lm_head_argmax_kernel(const __g
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer
-    if (lane == 0) {
+    {  // the whole warp, converged
+      const uint32_t leader = tc::elect_one();
       const uint64_t ad0 = tc::smem_desc_sw128(a_s(0), 16, 1024);
       const uint64_t bd0 = tc::smem_desc_sw128(b_s(0), 16, 1024);
+      // a wait's answer is the warp's: the lanes stay together
+      auto wait = [&](uint32_t bar, int parity) {
+        return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, abort_flag, wait_ns)) != 0;
+      };
       int64_t g = 0;
       int it = 0;  // tiles of this CTA
       int nd = 0;  // commits that a final wait covers
@@ -141,15 +146,15 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lm_head_argmax_kernel(const __g
       for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++it) {
         const int ab = it & 1;
         // the epilogue has read this accumulator's previous tile
-        if (it >= 2 && !tc::mbar_wait(te0 + 8 * ab, ((it >> 1) - 1) & 1, abort_flag, wait_ns)) {
-          give_up();
+        if (it >= 2 && !wait(te0 + 8 * ab, ((it >> 1) - 1) & 1)) {
+          if (leader) give_up();
           break;
         }
         tc::fence_after_sync();
         for (int kb = 0; kb < nk; ++kb, ++g) {
           const int st = int(g % STAGES);
-          if (!tc::mbar_wait(full0 + 8 * st, (g / STAGES) & 1, abort_flag, wait_ns)) {
-            give_up();
+          if (!wait(full0 + 8 * st, (g / STAGES) & 1)) {
+            if (leader) give_up();
             ok = false;
             break;
           }
@@ -158,11 +163,11 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lm_head_argmax_kernel(const __g
           for (int k = 0; k < BK / 16; ++k) {
             const uint32_t off = k * 32;  // 16 bf16 along K
             tc::mma_ss(tmem + 256u * ab, ad0 + ((uint32_t(st) * A_STAGE + off) >> 4),
-                       bd0 + ((uint32_t(st) * B_STAGE + off) >> 4), IDESC, (kb > 0 || k > 0) ? 1u : 0u);
+                       bd0 + ((uint32_t(st) * B_STAGE + off) >> 4), IDESC, (kb > 0 || k > 0) ? 1u : 0u, leader);
           }
-          tc::mma_commit(empty0 + 8 * st);
+          tc::mma_commit(empty0 + 8 * st, leader);
         }
-        tc::mma_commit(tf0 + 8 * ab);
+        tc::mma_commit(tf0 + 8 * ab, leader);
         ++nd;
       }
       // every MMA has completed before TMEM is freed
