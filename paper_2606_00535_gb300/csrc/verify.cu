@@ -928,6 +928,7 @@ struct StepParams {
   TreeParams tr;
   KVParams kv;
   int32_t max_path;
+  int32_t ntail;  // CTAs per sequence of the walk and compaction launch
   int32_t *pred;  // [B, T_max] predictions (caller's argmax_out or workspace)
   bool pred_in_ws;
   int32_t *accept_len, *path, *out_tokens, *new_kv_len;
@@ -991,14 +992,20 @@ __global__ void __launch_bounds__(256) verify_sample_select_kernel(const StepPar
   if ((threadIdx.x & 31) == 0) p.pred[r] = idx;
 }
 
-// Launch 2 of the verification tail, one CTA per sequence, chained to launch 1
-// by programmatic dependent launch (it may start early and waits until launch
-// 1 has completed): the acceptance walk, its outputs, and the KV compaction.
+// Launch 2 of the verification tail, p.ntail CTAs per sequence, chained to
+// launch 1 by programmatic dependent launch (it may start early and waits
+// until launch 1 has completed): the acceptance walk, its outputs, and the KV
+// compaction. Every CTA of a sequence does the same walk (a warp's work on 64
+// predictions); the first writes the outputs, and the compaction's 16-byte
+// columns, of which a whole model's cache has thousands, are spread over all
+// of them: the moves are latency-bound, so one CTA going through the columns
+// of 32 layers x 32 heads took 50 us where the spread takes the time of one
+// batch of moves (see tail_ctas for the sizes).
 __global__ void __launch_bounds__(TAIL_THREADS) verify_tail_kernel(const StepParams p) {
   __shared__ int32_t s_path[65], s_out[65], s_pg[2];
   __shared__ int64_t s_src[65], s_dst[65];
   __shared__ int s_n;
-  const int b = blockIdx.x, Tm = p.tr.T_max;
+  const int b = blockIdx.x / p.ntail, part = blockIdx.x % p.ntail, Tm = p.tr.T_max;
   const int64_t rb = int64_t(b) * Tm;
   const int T = __ldg(p.tr.tree_len + b);
   const int L = __ldg(p.tr.kv_len + b);
@@ -1025,21 +1032,36 @@ __global__ void __launch_bounds__(TAIL_THREADS) verify_tail_kernel(const StepPar
     else w = tree_walk_finish(ts, p.pred + rb, T, p.max_path, s_path, s_out);
     if (w.bad) {
       w.n = -1;
-      if (threadIdx.x == 0) flag(p.status, w.bad);
+      if (part == 0 && threadIdx.x == 0) flag(p.status, w.bad);
     }
-    write_walk(b, w.n, L, p.tr.tokens + rb, p.pred + rb, s_path, p.max_path, p.accept_len, p.path, p.out_tokens,
-               p.new_kv_len, s_out);
-    if (p.pred_in_ws && T >= 1 && T <= Tm) {  // leave the workspace zero-filled
+    if (part == 0)
+      write_walk(b, w.n, L, p.tr.tokens + rb, p.pred + rb, s_path, p.max_path, p.accept_len, p.path, p.out_tokens,
+                 p.new_kv_len, s_out);
+    if (p.pred_in_ws && T >= 1 && T <= Tm) {
+      // leave the workspace zero-filled: the CTA that read the predictions
+      // last (a count on the sequence's first row counter, zero again since
+      // the argmax grid completed) clears them
+      int last = 1;
+      if (p.ntail > 1) {
+        __threadfence();
+        __syncwarp();
+        if (threadIdx.x == 0) {
+          last = atomicAdd(p.am.cnt + rb, 1) == p.ntail - 1;
+          if (last) p.am.cnt[rb] = 0;
+        }
+        last = __shfl_sync(0xffffffffu, last, 0);
+      }
       __syncwarp();
-      for (int x = threadIdx.x; x < T; x += 32) p.pred[rb + x] = 0;
+      for (int x = threadIdx.x; last && x < T; x += 32) p.pred[rb + x] = 0;
     }
     bool ok = w.n > 0;
-    if (ok) ok = move_offsets(p.kv, b, L, w.n, s_path, s_src, s_dst, p.status, s_pg);
+    if (ok) ok = move_offsets(p.kv, b, L, w.n, s_path, s_src, s_dst, part == 0 ? p.status : nullptr, s_pg);
     if (threadIdx.x == 0) s_n = ok ? w.n : 0;
   }
   __syncthreads();
   const int n = s_n;
-  if (n > 0) compact_units(p.kv, n, s_src, s_dst, threadIdx.x, blockDim.x);
+  if (n > 0)
+    compact_units(p.kv, n, s_src, s_dst, part * int64_t(blockDim.x) + threadIdx.x, int64_t(p.ntail) * blockDim.x);
 }
 
 // ------------------------------------------------------------------ speculative sampling
@@ -1711,6 +1733,17 @@ dreams_status_t launch_dependent(void (*kernel)(Args...), dim3 grid, dim3 block,
   return check_launch();
 }
 
+// CTAs per sequence of the walk and compaction: one thread per 16-byte column
+// of the cache (all layers, K and V, all heads), while the batch's CTAs stay
+// within about four per SM, so that they are resident early next to the argmax
+// grid. One layer of 8 heads (256 columns) is one CTA; 32 layers of 32 heads
+// (32768 columns) for one sequence are 128.
+inline int32_t tail_ctas(const KVParams &kv, int64_t B) {
+  const int64_t units = int64_t(2) * kv.n_layers * kv.Hkv * kv.ch;
+  const int64_t most = std::max<int64_t>(1, 4 * int64_t(num_sms()) / B);
+  return int32_t(std::max<int64_t>(1, std::min<int64_t>((units + TAIL_THREADS - 1) / TAIL_THREADS, most)));
+}
+
 // CTAs per sequence of the speculative walk (a power of two): the fewest whose
 // slices of at most SPEC_MAX_J chunks cover V, doubled while every CTA keeps a
 // chunk of the vocabulary and the batch leaves SMs idle: up to 8, or 16 for
@@ -1887,6 +1920,7 @@ extern "C" dreams_status_t dreams_verify_step(const void *logits, dreams_dtype_t
   int32_t *ws_pred = reinterpret_cast<int32_t *>(ws + argmax_ws(rows));
   p.pred = argmax_out != nullptr ? argmax_out : ws_pred;
   p.pred_in_ws = argmax_out == nullptr;
+  p.ntail = tail_ctas(p.kv, tree->B);
   p.max_path = max_path;
   p.accept_len = accept_len;
   p.path = path;
@@ -1899,21 +1933,7 @@ extern "C" dreams_status_t dreams_verify_step(const void *logits, dreams_dtype_t
   else verify_rows_kernel<__nv_bfloat16><<<grid, ARGMAX_THREADS, 0, s>>>(p);
   dreams_status_t st = check_launch();
   if (st != DREAMS_OK) return st;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned(tree->B));
-  cfg.blockDim = dim3(TAIL_THREADS);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, verify_tail_kernel, p);
-  if (e != cudaSuccess) {
-    set_last_cuda_error(e);
-    return DREAMS_ERR_CUDA;
-  }
-  return check_launch();
+  return launch_dependent(verify_tail_kernel, dim3(unsigned(tree->B * p.ntail)), dim3(TAIL_THREADS), s, p);
 }
 
 extern "C" size_t dreams_vocab_sample_workspace_size(int64_t rows, int64_t V) {
@@ -1979,6 +1999,7 @@ extern "C" dreams_status_t dreams_verify_step_sampled(
   int32_t *ws_pred = reinterpret_cast<int32_t *>(ws + sample_ws(rows, V));
   p.pred = sample_out != nullptr ? sample_out : ws_pred;
   p.pred_in_ws = false;
+  p.ntail = tail_ctas(p.kv, tree->B);
   p.max_path = max_path;
   p.accept_len = accept_len;
   p.path = path;
@@ -1994,7 +2015,7 @@ extern "C" dreams_status_t dreams_verify_step_sampled(
   st = dtype == DREAMS_F32 ? launch_dependent(verify_sample_select_kernel<float>, g2, dim3(256), s, p)
                            : launch_dependent(verify_sample_select_kernel<__nv_bfloat16>, g2, dim3(256), s, p);
   if (st != DREAMS_OK) return st;
-  return launch_dependent(verify_tail_kernel, dim3(unsigned(tree->B)), dim3(TAIL_THREADS), s, p);
+  return launch_dependent(verify_tail_kernel, dim3(unsigned(tree->B * p.ntail)), dim3(TAIL_THREADS), s, p);
 }
 
 extern "C" dreams_status_t dreams_verify_step_speculative(
