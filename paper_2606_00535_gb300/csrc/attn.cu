@@ -191,7 +191,8 @@ __device__ __forceinline__ int split_tiles(const AttnParams &p, int b, int s) {
 // first (a counting sort; pairs of equal size may come in any order, which
 // changes only which SM computes them, not the result).
 __global__ void __launch_bounds__(ORDER_THREADS) tree_attn_order_kernel(const AttnParams p) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  grid_wait();
+  launch_successor();
   __shared__ int bucket[ORDER_KEYS];
   __shared__ int warp_sum[ORDER_THREADS / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -274,6 +275,8 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_c
   __shared__ int s_key[RANK_PAIRS];
   __shared__ int s_pair;
 
+  grid_wait();
+  launch_successor();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int per_pair = p.Hkv * p.nrb;
   const int pair_pos = blockIdx.x / per_pair;
@@ -288,8 +291,7 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_c
   const int rb = causal ? p.nrb - 1 - gr / p.Hkv : gr - g * p.nrb;
   int pair = pair_pos;
   if (p.order != nullptr) {
-    // the order comes from the preceding kernel (programmatic dependent launch)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // the order comes from the preceding kernel
     pair = __ldcg(p.order + pair_pos);
   } else if (p.rank) {
     // few pairs: the CTA takes the pair of rank pair_pos in the order by KV
@@ -1065,7 +1067,6 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_c
     tc::fence_after_sync();
     tc::tmem_dealloc(tmem, TMEM_COLS);
   }
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Log-sum-exp merge of the split partials: one warp per query row of a
@@ -1077,7 +1078,8 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_c
 // once that grid has completed and its writes are visible.
 template <int D, bool ENT>
 __global__ void __launch_bounds__(256) tree_attn_merge_kernel(const AttnParams p) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  grid_wait();
+  launch_successor();
   constexpr int NL = D / 4;  // lanes holding 4 columns each
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t row = int64_t(blockIdx.x) * 8 + warp;
@@ -1280,32 +1282,16 @@ constexpr size_t smem_bytes() {
   return std::max<size_t>(size_t(D / 64) * ROWS * 128 + size_t(NK + NV) * (D / 64) * KT * 128 + 1024, 120 * 1024);
 }
 
-cudaError_t launch_pdl(const void *func, dim3 grid, dim3 block, size_t smem, cudaStream_t stream, bool pdl,
-                       void **args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  return cudaLaunchKernelExC(&cfg, func, args);
-}
-
 template <int D, bool ENT>
 dreams_status_t launch(const AttnParams &a, const AttnPlan &pl, const dreams_kv_cache_t *kv, const void *k,
                        const void *v, int B, int64_t q_stride_b, int64_t q_stride_t, cudaStream_t stream) {
   constexpr size_t smem = smem_bytes<D>();
-  const void *kernel =
-      a.mode == ATTN_CAUSAL
-          ? reinterpret_cast<const void *>(tree_attn_tc_kernel<D, ENT, false, false>)
-          : (kv->page_table != nullptr ? reinterpret_cast<const void *>(tree_attn_tc_kernel<D, ENT, true, true>)
-                                       : reinterpret_cast<const void *>(tree_attn_tc_kernel<D, ENT, true, false>));
+  void (*kernel)(const TcParams) =
+      a.mode == ATTN_CAUSAL ? tree_attn_tc_kernel<D, ENT, false, false>
+                            : (kv->page_table != nullptr ? tree_attn_tc_kernel<D, ENT, true, true>
+                                                         : tree_attn_tc_kernel<D, ENT, true, false>);
   {
-    const dreams_status_t st = ensure_max_dynamic_smem(kernel, int(smem));
+    const dreams_status_t st = ensure_max_dynamic_smem(reinterpret_cast<const void *>(kernel), int(smem));
     if (st != DREAMS_OK) return st;
   }
   TcParams P;
@@ -1318,29 +1304,14 @@ dreams_status_t launch(const AttnParams &a, const AttnPlan &pl, const dreams_kv_
                   int64_t(a.Hq) * D))
     return DREAMS_ERR_UNSUPPORTED;
   if (pl.ordered) {
-    tree_attn_order_kernel<<<1, ORDER_THREADS, 0, stream>>>(a);
-    dreams_status_t st = check_launch();
+    const dreams_status_t st = launch_kernel(tree_attn_order_kernel, dim3(1), dim3(ORDER_THREADS), 0, stream, a);
     if (st != DREAMS_OK) return st;
   }
   const int64_t ctas = int64_t(B) * pl.nsplit * a.Hkv * pl.nrb;
-  void *args_attn[] = {&P};
-  cudaError_t e = launch_pdl(kernel, dim3(unsigned(ctas)), dim3(THREADS), smem, stream, pl.ordered, args_attn);
-  if (e != cudaSuccess) {
-    set_last_cuda_error(e);
-    return DREAMS_ERR_CUDA;
-  }
-  dreams_status_t st = check_launch();
+  const dreams_status_t st = launch_kernel(kernel, dim3(unsigned(ctas)), dim3(THREADS), smem, stream, P);
   if (st != DREAMS_OK || pl.nsplit == 1) return st;
   const int64_t rows = int64_t(B) * a.Hkv * pl.nrb * ROWS;
-  AttnParams am = a;
-  void *args_merge[] = {&am};
-  e = launch_pdl(reinterpret_cast<const void *>(tree_attn_merge_kernel<D, ENT>), dim3(unsigned((rows + 7) / 8)),
-                 dim3(256), 0, stream, true, args_merge);
-  if (e != cudaSuccess) {
-    set_last_cuda_error(e);
-    return DREAMS_ERR_CUDA;
-  }
-  return check_launch();
+  return launch_kernel(tree_attn_merge_kernel<D, ENT>, dim3(unsigned((rows + 7) / 8)), dim3(256), 0, stream, a);
 }
 
 }  // namespace

@@ -35,6 +35,41 @@ inline dreams_status_t check_launch() {
   return DREAMS_OK;
 }
 
+// Every kernel of the library is launched as a programmatic dependent of the
+// launch before it on the stream: its CTAs may become resident while that grid
+// drains, and each begins with grid_wait(), which returns once that grid has
+// completed and its writes are visible. Each then lets its own successor start
+// (launch_successor, after the wait, so that at most one grid ahead of a
+// running CTA is unfinished). Between back-to-back calls this takes the launch
+// gap out. A kernel that reads global memory before its wait may read only
+// what its own predecessor's inputs were (the walk's tree arrays), and reads
+// it through L2 (__ldcg): L1 may hold older lines until the wait.
+template <typename... Params, typename... Args>
+dreams_status_t launch_kernel(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                              Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+  if (e != cudaSuccess) {
+    set_last_cuda_error(e);
+    return DREAMS_ERR_CUDA;
+  }
+  return check_launch();
+}
+
+// Waits until the preceding grid has completed and its writes are visible.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next launch on the stream start once every CTA has come here.
+__device__ __forceinline__ void launch_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 __device__ __forceinline__ void flag(int32_t *status_word, int32_t bits) {

@@ -96,6 +96,8 @@ __device__ __forceinline__ void add_words(const uint4 *w, float (&acc)[8]) {
 // Rows are loaded as raw 16-byte words, 32 words per thread in flight.
 template <typename T>
 __global__ void __launch_bounds__(MAX_PART_THREADS) importance_partial_kernel(const ImpParams p) {
+  grid_wait();
+  launch_successor();
   constexpr int WPG = int(sizeof(T)) / 2;  // words per 8-column group
   constexpr int U = 8 / WPG;               // rows in flight
   const int b = blockIdx.z, c = blockIdx.y;
@@ -142,7 +144,6 @@ __global__ void __launch_bounds__(MAX_PART_THREADS) importance_partial_kernel(co
     for (int i = 0; i < 8; ++i)
       if (i < n_left && col + i >= p.v0) out[col + i - p.v0] = acc[i];
   }
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Block-wide exclusive prefix sum of one int per thread (SEL_THREADS threads);
@@ -178,8 +179,8 @@ __device__ int block_exclusive_scan(int v, int &total) {
 // row-range partials / (H Q). Thread (x, y) adds ranges y, y + 32, ... of
 // column x; the 32 sums meet in a fixed tree.
 __global__ void __launch_bounds__(1024) importance_reduce_kernel(const ImpParams p, float *importance) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  grid_wait();
+  launch_successor();
   __shared__ float red[32][33];
   const int b = blockIdx.y, tx = threadIdx.x, ty = threadIdx.y;
   const int64_t n = p.n_vis;
@@ -205,7 +206,8 @@ __global__ void __launch_bounds__(1024) importance_reduce_kernel(const ImpParams
 // order. s_key holds n_vis keys (dynamic shared memory).
 __global__ void __launch_bounds__(SEL_THREADS) importance_select_kernel(const ImpParams p, int32_t r,
                                                                         const float *importance, int32_t *keep) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  grid_wait();
+  launch_successor();
   extern __shared__ uint32_t s_key[];
   __shared__ int s_hist[256];
   __shared__ uint32_t s_prefix;
@@ -357,46 +359,14 @@ extern "C" dreams_status_t dreams_visual_importance(const void *attn, dreams_dty
   if (cblocks > INT_MAX || p.nchunk > 65535) return DREAMS_ERR_UNSUPPORTED;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const dim3 grid(unsigned(cblocks), unsigned(p.nchunk), unsigned(B));
-  if (dtype == DREAMS_F32) importance_partial_kernel<float><<<grid, tpb, 0, s>>>(p);
-  else importance_partial_kernel<__nv_bfloat16><<<grid, tpb, 0, s>>>(p);
-  dreams_status_t st = check_launch();
+  dreams_status_t st = dtype == DREAMS_F32 ? launch_kernel(importance_partial_kernel<float>, grid, dim3(tpb), 0, s, p)
+                                           : launch_kernel(importance_partial_kernel<__nv_bfloat16>, grid, dim3(tpb), 0, s, p);
   if (st != DREAMS_OK) return st;
-  {
-    cudaLaunchConfig_t rc = {};
-    rc.gridDim = dim3(unsigned((n_vis + 31) / 32), unsigned(B));
-    rc.blockDim = dim3(32, 32);
-    rc.stream = s;
-    cudaLaunchAttribute ra[1];
-    ra[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    ra[0].val.programmaticStreamSerializationAllowed = 1;
-    rc.attrs = ra;
-    rc.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&rc, importance_reduce_kernel, p, importance);
-    if (e != cudaSuccess) {
-      set_last_cuda_error(e);
-      return DREAMS_ERR_CUDA;
-    }
-    st = check_launch();
-    if (st != DREAMS_OK) return st;
-  }
-  const size_t smem = size_t(n_vis) * 4;
+  st = launch_kernel(importance_reduce_kernel, dim3(unsigned((n_vis + 31) / 32), unsigned(B)), dim3(32, 32), 0, s, p,
+                     importance);
+  if (st != DREAMS_OK) return st;
   st = ensure_max_dynamic_smem(reinterpret_cast<const void *>(importance_select_kernel), 48 * 1024 * 4);
   if (st != DREAMS_OK) return st;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned(B));
-  cfg.blockDim = dim3(SEL_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t e =
-      cudaLaunchKernelEx(&cfg, importance_select_kernel, p, r, static_cast<const float *>(importance), keep);
-  if (e != cudaSuccess) {
-    set_last_cuda_error(e);
-    return DREAMS_ERR_CUDA;
-  }
-  return check_launch();
+  return launch_kernel(importance_select_kernel, dim3(unsigned(B)), dim3(SEL_THREADS), size_t(n_vis) * 4, s, p, r,
+                       importance, keep);
 }

@@ -88,6 +88,8 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lm_head_argmax_kernel(const __g
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = s_tmem;
+  grid_wait();
+  launch_successor();
   volatile int *abort_flag = &s_abort;
   const uint64_t wait_ns = P.wait_ns;
   auto give_up = [&]() {
@@ -234,7 +236,6 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lm_head_argmax_kernel(const __g
     tc::fence_after_sync();
     tc::tmem_dealloc(tmem, 512);
   }
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // The row's index (and its maximum value) from its slot; resets the slot. A
@@ -242,7 +243,8 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lm_head_argmax_kernel(const __g
 // candidate, and no (key, index) pair packs to 0) leaves the row untouched.
 __global__ void __launch_bounds__(256) lm_head_finish_kernel(unsigned long long *slot, int64_t rows, int32_t *out_idx,
                                                              float *out_max) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  grid_wait();
+  launch_successor();
   const int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (r >= rows) return;
   const unsigned long long v = slot[r];
@@ -320,22 +322,8 @@ extern "C" dreams_status_t dreams_lm_head_argmax(const void *hidden, int64_t row
   const int64_t ntiles = int64_t(P.nm) * P.nn;
   const unsigned grid = unsigned(std::min<int64_t>(ntiles, num_sms()));
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  lm_head_argmax_kernel<0><<<grid, LM_THREADS, LM_SMEM, s>>>(P);
-  dreams_status_t st = check_launch();
+  const dreams_status_t st = launch_kernel(lm_head_argmax_kernel<0>, dim3(grid), dim3(LM_THREADS), LM_SMEM, s, P);
   if (st != DREAMS_OK) return st;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned((rows + 255) / 256));
-  cfg.blockDim = dim3(256);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, lm_head_finish_kernel, P.slot, rows, out_idx, out_max);
-  if (e != cudaSuccess) {
-    set_last_cuda_error(e);
-    return DREAMS_ERR_CUDA;
-  }
-  return check_launch();
+  return launch_kernel(lm_head_finish_kernel, dim3(unsigned((rows + 255) / 256)), dim3(256), 0, s, P.slot, rows, out_idx,
+                       out_max);
 }

@@ -225,6 +225,8 @@ struct ArgmaxParams {
 
 template <typename T>
 __global__ void __launch_bounds__(ARGMAX_THREADS) vocab_argmax_kernel(const ArgmaxParams p) {
+  grid_wait();
+  launch_successor();
   const int64_t row = blockIdx.x / p.nchunk;
   const int c = blockIdx.x % p.nchunk;
   const T *base = static_cast<const T *>(p.logits) + row * p.row_stride;
@@ -602,19 +604,20 @@ __device__ int sample_select_warp(const SampleParams &p, const T *row, const flo
 
 template <typename T>
 __global__ void __launch_bounds__(SAMPLE_THREADS, sizeof(T) == 2 ? 6 : 4) vocab_sample_stats_kernel(const SampleParams p) {
+  grid_wait();
+  launch_successor();
   const int64_t r = blockIdx.x / p.ncta_row;
   const int c = blockIdx.x % p.ncta_row;
   const int64_t g0 = int64_t(c) * p.seg_per_cta, g1 = std::min<int64_t>(p.nseg, g0 + p.seg_per_cta);
   sample_stats<T>(p, static_cast<const T *>(p.logits) + r * p.row_stride, p.seg + r * p.nseg, g0, g1);
-  // the selection grid may launch as this one drains
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Stage 2, one warp per row, chained to stage 1 by programmatic dependent
 // launch (it waits until stage 1 has completed).
 template <typename T>
 __global__ void __launch_bounds__(256) vocab_sample_select_kernel(const SampleParams p, int64_t rows, int32_t *out) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  grid_wait();
+  launch_successor();
   const int64_t r = int64_t(blockIdx.x) * 8 + (threadIdx.x >> 5);
   if (r >= rows) return;
   const int idx = sample_select_warp<T>(p, static_cast<const T *>(p.logits) + r * p.row_stride, p.seg + r * p.nseg,
@@ -648,8 +651,8 @@ __device__ TreeShape tree_shape_warp(const int32_t *par_row, const int32_t *tok_
   for (int h = 0; h < 2; ++h) {
     const int i = lane + 32 * h;
     const bool live = i < T;
-    ts.par[h] = live ? __ldg(par_row + i) : -1;
-    ts.tok[h] = live ? __ldg(tok_row + i) : 0;
+    ts.par[h] = live ? __ldcg(par_row + i) : -1;
+    ts.tok[h] = live ? __ldcg(tok_row + i) : 0;
     if (i == 0) bad |= (ts.par[h] != -1);
     else if (live) bad |= (ts.par[h] < 0 || ts.par[h] >= i);
   }
@@ -867,6 +870,8 @@ struct TreeParams {
 __global__ void __launch_bounds__(32) accept_path_kernel(const int32_t *pred, const TreeParams tr, int max_path,
                                                          int32_t *accept_len, int32_t *path, int32_t *out_tokens,
                                                          int32_t *new_kv_len, int32_t *status) {
+  grid_wait();
+  launch_successor();
   __shared__ int32_t s_path[65];
   const int b = blockIdx.x;
   const int T = __ldg(tr.tree_len + b), L = __ldg(tr.kv_len + b);
@@ -885,6 +890,8 @@ __global__ void __launch_bounds__(32) accept_path_kernel(const int32_t *pred, co
 __global__ void __launch_bounds__(TAIL_THREADS) kv_compact_kernel(const KVParams kv, const int32_t *kv_len,
                                                                   const int32_t *accept_len, const int32_t *path,
                                                                   int max_path, int32_t *status) {
+  grid_wait();
+  launch_successor();
   __shared__ int32_t s_path[65];
   __shared__ int64_t s_src[65], s_dst[65];
   __shared__ int s_ok;
@@ -940,8 +947,8 @@ struct StepParams {
 // that completes a node's row writes the node's prediction.
 template <typename T>
 __global__ void __launch_bounds__(ARGMAX_THREADS) verify_rows_kernel(const StepParams p) {
-  // the walk kernel may start now: it waits for this grid to complete
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  grid_wait();
+  launch_successor();  // the walk kernel: it waits for this grid to complete
   const int nchunk = p.am.nchunk;
   const int c = blockIdx.x % nchunk;
   const int rowg = blockIdx.x / nchunk;
@@ -963,6 +970,8 @@ __global__ void __launch_bounds__(ARGMAX_THREADS) verify_rows_kernel(const StepP
 // which writes the draws as the predictions.
 template <typename T>
 __global__ void __launch_bounds__(SAMPLE_THREADS, sizeof(T) == 2 ? 6 : 4) verify_sample_stats_kernel(const StepParams p) {
+  grid_wait();
+  launch_successor();
   const int ncta = p.sp.ncta_row;
   const int rowg = blockIdx.x / ncta;
   const int b = rowg / p.tr.T_max, i = rowg % p.tr.T_max;
@@ -974,13 +983,12 @@ __global__ void __launch_bounds__(SAMPLE_THREADS, sizeof(T) == 2 ? 6 : 4) verify
     sample_stats<T>(p.sp, static_cast<const T *>(p.sp.logits) + r * p.sp.row_stride, p.sp.seg + r * p.sp.nseg,
                     g0, g1);
   }
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 template <typename T>
 __global__ void __launch_bounds__(256) verify_sample_select_kernel(const StepParams p) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  grid_wait();
+  launch_successor();
   const int rowg = blockIdx.x * 8 + (threadIdx.x >> 5);
   const int b = rowg / p.tr.T_max, i = rowg % p.tr.T_max;
   if (b >= p.tr.B) return;
@@ -1007,8 +1015,8 @@ __global__ void __launch_bounds__(TAIL_THREADS) verify_tail_kernel(const StepPar
   __shared__ int s_n;
   const int b = blockIdx.x / p.ntail, part = blockIdx.x % p.ntail, Tm = p.tr.T_max;
   const int64_t rb = int64_t(b) * Tm;
-  const int T = __ldg(p.tr.tree_len + b);
-  const int L = __ldg(p.tr.kv_len + b);
+  const int T = __ldcg(p.tr.tree_len + b);
+  const int L = __ldcg(p.tr.kv_len + b);
   // Everything that needs no prediction is done while the argmax grid runs:
   // the tree's shape (with its tokens, which the walk then emits from
   // registers) and, for a paged cache, the page-table entries of the tree's
@@ -1019,11 +1027,12 @@ __global__ void __launch_bounds__(TAIL_THREADS) verify_tail_kernel(const StepPar
     const int lane = threadIdx.x;
     int e = -1;
     if (lane < 2 && lens_ok && p.kv.page_table != nullptr && (L >> 6) + lane < p.kv.pages_per_seq)
-      e = __ldg(p.kv.page_table + int64_t(b) * p.kv.pages_per_seq + (L >> 6) + lane);
+      e = __ldcg(p.kv.page_table + int64_t(b) * p.kv.pages_per_seq + (L >> 6) + lane);
     if (lens_ok) ts = tree_shape_warp(p.tr.parent + rb, p.tr.tokens + rb, T);
     if (lane < 2) s_pg[lane] = e;
   }
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  grid_wait();
+  launch_successor();
   if (threadIdx.x < 32) {
     WalkOut w{-1, 0};
     if (T < 1 || T > Tm) w.bad = DREAMS_DATA_BAD_TREE_LEN;
@@ -1472,6 +1481,8 @@ __device__ int spec_slice_draw(SpecShared &sh, const float *et, const float *ed,
 // decisions, the bonus draw, the outputs and the KV compaction.
 template <typename T>
 __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParams p) {
+  grid_wait();
+  launch_successor();
   extern __shared__ __align__(16) float spec_dyn[];
   __shared__ SpecShared sh;
   const int cs = p.cs, J = p.J;
@@ -1713,26 +1724,6 @@ SamplePlan plan_sample(int64_t rows, int64_t V) {
 
 size_t sample_ws(int64_t rows, int64_t V) { return align_up(size_t(rows) * size_t((V + SEG - 1) / SEG) * 8, 256); }
 
-// Launches `kernel` as a programmatic dependent of the previous launch on the stream.
-template <typename... Args>
-dreams_status_t launch_dependent(void (*kernel)(Args...), dim3 grid, dim3 block, cudaStream_t s, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
-  if (e != cudaSuccess) {
-    set_last_cuda_error(e);
-    return DREAMS_ERR_CUDA;
-  }
-  return check_launch();
-}
-
 // CTAs per sequence of the walk and compaction: one thread per 16-byte column
 // of the cache (all layers, K and V, all heads), while the batch's CTAs stay
 // within about four per SM, so that they are resident early next to the argmax
@@ -1852,9 +1843,8 @@ extern "C" dreams_status_t dreams_vocab_argmax(const void *logits, dreams_dtype_
   }
   const dim3 grid(unsigned(rows * pl.nchunk));
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (dtype == DREAMS_F32) vocab_argmax_kernel<float><<<grid, ARGMAX_THREADS, 0, s>>>(p);
-  else vocab_argmax_kernel<__nv_bfloat16><<<grid, ARGMAX_THREADS, 0, s>>>(p);
-  return check_launch();
+  return dtype == DREAMS_F32 ? launch_kernel(vocab_argmax_kernel<float>, grid, dim3(ARGMAX_THREADS), 0, s, p)
+                           : launch_kernel(vocab_argmax_kernel<__nv_bfloat16>, grid, dim3(ARGMAX_THREADS), 0, s, p);
 }
 
 extern "C" dreams_status_t dreams_accept_path(const int32_t *argmax, const dreams_tree_t *tree, int32_t max_path,
@@ -1864,9 +1854,8 @@ extern "C" dreams_status_t dreams_accept_path(const int32_t *argmax, const dream
   if (argmax == nullptr || !tree_params(tree, true, tr) || max_path < 1 || accept_len == nullptr ||
       path == nullptr || out_tokens == nullptr || new_kv_len == nullptr)
     return DREAMS_ERR_INVALID_ARG;
-  accept_path_kernel<<<tree->B, 32, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-      argmax, tr, max_path, accept_len, path, out_tokens, new_kv_len, status_word);
-  return check_launch();
+  return launch_kernel(accept_path_kernel, dim3(unsigned(tree->B)), dim3(32), 0, reinterpret_cast<cudaStream_t>(stream),
+                       argmax, tr, max_path, accept_len, path, out_tokens, new_kv_len, status_word);
 }
 
 extern "C" dreams_status_t dreams_kv_compact(const dreams_kv_cache_t *kv, int32_t B, const int32_t *kv_len,
@@ -1878,9 +1867,8 @@ extern "C" dreams_status_t dreams_kv_compact(const dreams_kv_cache_t *kv, int32_
     return DREAMS_ERR_INVALID_ARG;
   const int64_t units = int64_t(2) * kv->n_layers * kv->Hkv * (kv->D / 8);
   const int64_t blocks = std::min<int64_t>((units + TAIL_THREADS - 1) / TAIL_THREADS, 1024);
-  kv_compact_kernel<<<dim3(unsigned(blocks), B), TAIL_THREADS, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-      kp, kv_len, accept_len, path, max_path, status_word);
-  return check_launch();
+  return launch_kernel(kv_compact_kernel, dim3(unsigned(blocks), B), dim3(TAIL_THREADS), 0,
+                       reinterpret_cast<cudaStream_t>(stream), kp, kv_len, accept_len, path, max_path, status_word);
 }
 
 extern "C" size_t dreams_verify_step_workspace_size(const dreams_tree_t *tree, int64_t V) {
@@ -1929,11 +1917,10 @@ extern "C" dreams_status_t dreams_verify_step(const void *logits, dreams_dtype_t
   p.status = status_word;
   const dim3 grid(unsigned(rows * pl.nchunk));
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (dtype == DREAMS_F32) verify_rows_kernel<float><<<grid, ARGMAX_THREADS, 0, s>>>(p);
-  else verify_rows_kernel<__nv_bfloat16><<<grid, ARGMAX_THREADS, 0, s>>>(p);
-  dreams_status_t st = check_launch();
+  dreams_status_t st = dtype == DREAMS_F32 ? launch_kernel(verify_rows_kernel<float>, grid, dim3(ARGMAX_THREADS), 0, s, p)
+                           : launch_kernel(verify_rows_kernel<__nv_bfloat16>, grid, dim3(ARGMAX_THREADS), 0, s, p);
   if (st != DREAMS_OK) return st;
-  return launch_dependent(verify_tail_kernel, dim3(unsigned(tree->B * p.ntail)), dim3(TAIL_THREADS), s, p);
+  return launch_kernel(verify_tail_kernel, dim3(unsigned(tree->B * p.ntail)), dim3(TAIL_THREADS), 0, s, p);
 }
 
 extern "C" size_t dreams_vocab_sample_workspace_size(int64_t rows, int64_t V) {
@@ -1960,12 +1947,11 @@ extern "C" dreams_status_t dreams_vocab_sample(const void *logits, dreams_dtype_
   if (ctas > INT_MAX || (rows + 7) / 8 > INT_MAX) return DREAMS_ERR_UNSUPPORTED;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const dim3 grid(static_cast<unsigned>(ctas)), g2(static_cast<unsigned>((rows + 7) / 8));
-  if (dtype == DREAMS_F32) vocab_sample_stats_kernel<float><<<grid, SAMPLE_THREADS, 0, s>>>(p);
-  else vocab_sample_stats_kernel<__nv_bfloat16><<<grid, SAMPLE_THREADS, 0, s>>>(p);
-  dreams_status_t st = check_launch();
+  dreams_status_t st = dtype == DREAMS_F32 ? launch_kernel(vocab_sample_stats_kernel<float>, grid, dim3(SAMPLE_THREADS), 0, s, p)
+                                           : launch_kernel(vocab_sample_stats_kernel<__nv_bfloat16>, grid, dim3(SAMPLE_THREADS), 0, s, p);
   if (st != DREAMS_OK) return st;
-  if (dtype == DREAMS_F32) return launch_dependent(vocab_sample_select_kernel<float>, g2, dim3(256), s, p, rows, out_idx);
-  return launch_dependent(vocab_sample_select_kernel<__nv_bfloat16>, g2, dim3(256), s, p, rows, out_idx);
+  if (dtype == DREAMS_F32) return launch_kernel(vocab_sample_select_kernel<float>, g2, dim3(256), 0, s, p, rows, out_idx);
+  return launch_kernel(vocab_sample_select_kernel<__nv_bfloat16>, g2, dim3(256), 0, s, p, rows, out_idx);
 }
 
 extern "C" size_t dreams_verify_step_sampled_workspace_size(const dreams_tree_t *tree, int64_t V) {
@@ -2008,14 +1994,13 @@ extern "C" dreams_status_t dreams_verify_step_sampled(
   p.status = status_word;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const dim3 grid(static_cast<unsigned>(ctas)), g2(static_cast<unsigned>((rows + 7) / 8));
-  if (dtype == DREAMS_F32) verify_sample_stats_kernel<float><<<grid, SAMPLE_THREADS, 0, s>>>(p);
-  else verify_sample_stats_kernel<__nv_bfloat16><<<grid, SAMPLE_THREADS, 0, s>>>(p);
-  dreams_status_t st = check_launch();
+  dreams_status_t st = dtype == DREAMS_F32 ? launch_kernel(verify_sample_stats_kernel<float>, grid, dim3(SAMPLE_THREADS), 0, s, p)
+                                           : launch_kernel(verify_sample_stats_kernel<__nv_bfloat16>, grid, dim3(SAMPLE_THREADS), 0, s, p);
   if (st != DREAMS_OK) return st;
-  st = dtype == DREAMS_F32 ? launch_dependent(verify_sample_select_kernel<float>, g2, dim3(256), s, p)
-                           : launch_dependent(verify_sample_select_kernel<__nv_bfloat16>, g2, dim3(256), s, p);
+  st = dtype == DREAMS_F32 ? launch_kernel(verify_sample_select_kernel<float>, g2, dim3(256), 0, s, p)
+                           : launch_kernel(verify_sample_select_kernel<__nv_bfloat16>, g2, dim3(256), 0, s, p);
   if (st != DREAMS_OK) return st;
-  return launch_dependent(verify_tail_kernel, dim3(unsigned(tree->B * p.ntail)), dim3(TAIL_THREADS), s, p);
+  return launch_kernel(verify_tail_kernel, dim3(unsigned(tree->B * p.ntail)), dim3(TAIL_THREADS), 0, s, p);
 }
 
 extern "C" dreams_status_t dreams_verify_step_speculative(
@@ -2071,13 +2056,15 @@ extern "C" dreams_status_t dreams_verify_step_speculative(
   cfg.blockDim = dim3(SPEC_THREADS);
   cfg.dynamicSmemBytes = size_t(smem);
   cfg.stream = reinterpret_cast<cudaStream_t>(stream);
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = unsigned(pl.cs);
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, p);
   if (e != cudaSuccess) {
     set_last_cuda_error(e);
@@ -2161,7 +2148,6 @@ extern "C" dreams_status_t dreams_vocab_argmax_noalloc(const void *logits, dream
     }
   }
   const dim3 grid(unsigned(rows * pl.nchunk));
-  if (dtype == DREAMS_F32) vocab_argmax_kernel<float><<<grid, ARGMAX_THREADS, 0, s>>>(p);
-  else vocab_argmax_kernel<__nv_bfloat16><<<grid, ARGMAX_THREADS, 0, s>>>(p);
-  return check_launch();
+  return dtype == DREAMS_F32 ? launch_kernel(vocab_argmax_kernel<float>, grid, dim3(ARGMAX_THREADS), 0, s, p)
+                           : launch_kernel(vocab_argmax_kernel<__nv_bfloat16>, grid, dim3(ARGMAX_THREADS), 0, s, p);
 }
