@@ -26,18 +26,15 @@
 //                       keeps V a tile behind K (QK^T of tile j + 1 runs
 //                       before PV of tile j); page-table entries are loaded
 //                       one tile ahead.
-//   warp 9, converged   MMA issuer (one elected lane's MMAs take effect): S = Q K^T (M128 N128, K-major operands) into
-//                       TMEM, O += P V (M128 N=D, P read from TMEM, V as an
-//                       MN-major operand). Tile j goes to warpgroup j % 2, and
-//                       the QK^T of tile j + 2 follows the PV of tile j (they
-//                       share that warpgroup's S/P columns). Per tile it
-//                       waits for P_j, then issues PV_j and QK_{j+2} (16
-//                       MMAs) under one commit.
-//                       Tree and cross-attention rows hand P_j over in two
-//                       halves of 64 keys, so the first half of PV_j runs
-//                       while the softmax finishes the tile; on a paged cache
-//                       the thread also commits V_j's stage free right after
-//                       PV_j.
+//   warp 9, converged   MMA issuer (one elected lane's MMAs take effect):
+//                       S = Q K^T (M128 N128, K-major operands) into TMEM,
+//                       O += P V (M128 N=D, P read from TMEM, V as an MN-major
+//                       operand). Tile j goes to warpgroup j % 2, and the QK^T
+//                       of tile j + 2 follows the PV of tile j (they share that
+//                       warpgroup's S/P columns). P_j comes in two parts, so
+//                       that PV_j over the first keys runs while the softmax
+//                       finishes the tile. It waits for the copies itself, and
+//                       commits V_j's stage free right after PV_j.
 //   warps 0-3, 4-7      two softmax warpgroups, one query row per thread. A
 //                       warpgroup owns one S/P buffer and its own O in TMEM
 //                       (256 columns each), so the two alternate over the
@@ -48,25 +45,22 @@
 //                       exceeds it by 2^8 (and only then rescales its O), and
 //                       writes P as bf16 over S. Woken by the commit after
 //                       QK_j (which also covers PV_{j-2}), one thread
-//                       releases the K stage of tile j and (unless the MMA
-//                       thread did) the V stage of tile j - 2 to the
-//                       producer; before the warpgroup signals P_j (or its
-//                       first half) it waits for V_j and K_{j+2} (or V_j) to
-//                       land, so that the MMA thread needs no other wait.
-//                       Warps whose rows are all padding sit out.
+//                       releases the K stage of tile j to the producer. Warps
+//                       whose rows are all padding sit out.
 // At the end the two warpgroups combine their (m, l, O) by log-sum-exp. A
 // block whose rows all lie inside the tensor leaves through TMA stores of the
 // output staged in shared memory; other blocks write each row's half of the
 // columns with 16-byte stores: the output, or the split partials that a merge
-// kernel (chained by programmatic dependent launch) combines. Every mbarrier wait is bounded (2 s); on a
-// timeout the CTA flags DREAMS_DATA_TIMEOUT, drains its copies and MMAs, frees
-// its TMEM and exits. The workspace holds no state between calls.
+// kernel combines. Every mbarrier wait is bounded (2 s); on a timeout the CTA
+// flags DREAMS_DATA_TIMEOUT, drains its copies and MMAs, frees its TMEM and
+// exits. The workspace holds no state between calls.
 #include <cuda.h>
 #include <limits.h>
 #include <math.h>
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "tc.cuh"
@@ -244,17 +238,15 @@ __global__ void __launch_bounds__(ORDER_THREADS) tree_attn_order_kernel(const At
   }
 }
 
-// SPLIT: P is handed to the MMA thread in two halves, so that the first half
-// of PV_j runs while the softmax warps finish the tile (tree and
-// cross-attention rows, bound by the softmax-MMA chain), or whole (causal
-// rows, bound by the tensor pipe, where the extra wait between the PV halves
-// costs more than it saves). VREL (with SPLIT): a V stage goes back to the
-// producer as soon as its PV has completed (one more commit per tile) rather
-// than at the next wake-up of the softmax warps: worth it where the copies
-// land late, on paged caches. The host picks both by mode and cache layout.
-template <int D, bool ENT, bool SPLIT, bool VREL>
+// P goes to the MMA warp in two parts, so that PV_j over the first keys runs
+// while the softmax warps finish the tile, and a V stage goes back to
+// the producer as soon as its PV has completed (a commit of its own). With the
+// MMAs issued by the converged warp an extra wait or commit hides under the
+// queued MMAs: both now pay on every path (causal prefill of 3392 tokens x 32
+// heads 115.7 -> 108.9 us a pass, batched trees 68.7 -> 64.5, a contiguous
+// cache of 3392 slots x 32 heads 18.7 -> 18.4).
+template <int D, bool ENT>
 __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_constant__ TcParams P) {
-  static_assert(SPLIT || !VREL, "the early V release goes with the two-half hand-off");
   const AttnParams &p = P.a;
   constexpr int NR = D / 64;                     // 128-byte column regions of a row
   constexpr uint32_t Q_REGION = ROWS * 128;      // 16 KB
@@ -263,6 +255,10 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_c
   constexpr uint32_t KV_TILE = NR * KV_REGION;   // one K or V tile
   constexpr uint32_t IDESC_QK = tc::idesc_bf16_f32(ROWS, KT, false);
   constexpr uint32_t IDESC_PV = tc::idesc_bf16_f32(ROWS, D, true);
+  // keys of a tile's first P hand-off: with the entropy sums the softmax is
+  // longer and 96 did better (prefill of 3392 tokens x 32 heads 103.2 against
+  // 106.5 us), without them 64 (3392 slots x 32 heads 18.0 against 18.3 us)
+  constexpr int FIRST = ENT ? 96 : 64;
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -421,8 +417,8 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_c
     if (!early) init_copy_barriers();
     for (int i = 0; i < 2; ++i) {
       tc::mbar_init(bs0 + 8 * i, 1);
-      tc::mbar_init(bp0 + 8 * i, 32 * n_act);
-      tc::mbar_init(bph0 + 8 * i, 32 * n_act);
+      tc::mbar_init(bp0 + 8 * i, n_act);  // one arrival per active warp
+      tc::mbar_init(bph0 + 8 * i, n_act);
     }
     tc::mbar_init(bdrain, 1);
     tc::mbar_init(bnever, 1);  // nothing arrives on it (the stall test hook waits on it)
@@ -614,12 +610,14 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_c
       const uint64_t qd0 = tc::smem_desc_sw128(q_s, 16, 1024);
       const uint64_t kd0 = tc::smem_desc_sw128(k_s(0), 16, 1024);
       const uint64_t vd0 = tc::smem_desc_sw128(v_s(0), KV_REGION, 1024);
-      // Per tile the warp takes one wait, then issues PV_j and QK_{j+2} (16
-      // MMAs) under one commit (with SPLIT, one wait before each half of
-      // PV_j). Issued by the converged warp, so that the operands stay in
-      // uniform registers (tc.cuh): batched serving (16 sequences, 32 q / 8 KV
-      // heads, 1500-6000 slots) 77.5 -> 70.0 us a pass, the causal prefill of
-      // 3392 tokens x 32 heads 122.9 -> 118.8 us.
+      // The MMAs are issued by the converged warp, so that their operands stay
+      // in uniform registers (tc.cuh): batched serving (16 sequences, 32 q / 8
+      // KV heads, 1500-6000 slots) 77.5 -> 70.0 us a pass, the causal prefill
+      // of 3392 tokens x 32 heads 122.9 -> 118.8 us. Waits for P, V and K then
+      // hide under the MMAs that are queued: the softmax warps, whose chain of
+      // scores, exponents and hand-off bounds a tile, wait for no copy (64.8
+      // -> 62.6 and 109.8 -> 104.2 us of GPU time against a softmax thread
+      // that saw the copies land before it handed P over).
       // S_j = Q K_j^T into warpgroup (j % 2)'s S buffer
       auto qk = [&](int j) {
         const int ks = j % NK;
@@ -632,13 +630,13 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_c
           tc::mma_ss(tmem + scol, ad, bd, IDESC_QK, k > 0 ? 1u : 0u, leader);
         }
       };
-      // O_w += P_j V_j, w = j % 2, over the tile's first (h = 0) or last 64 keys
-      auto pv = [&](int j, int h) {
+      // O_w += P_j V_j, w = j % 2, over the tile's first FIRST keys or the others
+      auto pv = [&](int j, auto second) {
+        constexpr bool h = decltype(second)::value;
         const int w = j & 1, ii = j >> 1, vs = j % NV;
         const uint32_t scol = 256u * w, ocol = 256u * w + 128u;
 #pragma unroll
-        for (int kk = 0; kk < KT / 32; ++kk) {
-          const int ks = h * (KT / 32) + kk;
+        for (int ks = h ? FIRST / 16 : 0; ks < (h ? KT : FIRST) / 16; ++ks) {
           const uint64_t bd = vd0 + ((uint32_t(vs) * KV_TILE + ks * 2048) >> 4);
           tc::mma_ts(tmem + ocol, tmem + scol + ks * 8, bd, IDESC_PV, (ii > 0 || ks > 0) ? 1u : 0u, leader);
         }
@@ -663,29 +661,26 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_c
         }
       }
       // The commit after QK_{j+2} also covers PV_j (the pipe completes in
-      // order): the softmax warps, woken by it, release the stages of K_{j+2}
-      // and (without VREL) V_j to the producer.
+      // order): the softmax warps, woken by it, release the stage of K_{j+2}
+      // to the producer.
       for (int j = 0; j < ntiles && ok; ++j) {
         const int w = j & 1;
-        // P_j over the first 64 keys (the softmax warps arrive once one of
-        // them has also seen V_j land): its PV half runs while they finish
-        // the tile; then the rest of P_j (K_{j+2} landed as well). Without
-        // SPLIT, P_j whole.
-        if constexpr (SPLIT) {
-          ok = wait(bph0 + 8 * w, (j >> 1) & 1);
-          if (!ok) break;
-          tc::fence_after_sync();
-          pv(j, 0);
-        }
+        // P_j over its first keys: their PV runs while the softmax warps
+        // finish the tile; then the rest of P_j.
+        ok = wait(bph0 + 8 * w, (j >> 1) & 1) && wait(vf0 + 8 * (j % NV), (j / NV) & 1);
+        if (!ok) break;
+        tc::fence_after_sync();
+        pv(j, std::false_type{});
         ok = wait(bp0 + 8 * w, (j >> 1) & 1);
         if (!ok) break;
         tc::fence_after_sync();
-        if constexpr (!SPLIT) pv(j, 0);
-        pv(j, 1);
-        // with VREL, V_j's stage goes back to the producer as soon as PV_j
-        // has completed, ahead of QK_{j+2} (an arrival on its empty barrier)
-        if constexpr (VREL) tc::mma_commit(ve0 + 8 * (j % NV), leader);
+        pv(j, std::true_type{});
+        // V_j's stage goes back to the producer as soon as PV_j has completed,
+        // ahead of QK_{j+2} (an arrival on its empty barrier)
+        tc::mma_commit(ve0 + 8 * (j % NV), leader);
         if (j + 2 < ntiles) {
+          ok = kwait(j + 2);
+          if (!ok) break;
           qk(j + 2);
           tc::mma_commit(bs0 + 8 * w, leader);
         }
@@ -711,14 +706,10 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_c
         break;
       }
       // S_j is complete, and so (issued earlier) is this warpgroup's previous
-      // PV, so O may be rescaled below. The K stage of tile j and (unless the
-      // MMA thread's commit already did, VREL) the V stage of tile j - 2, read
-      // by that PV, go back to the producer.
+      // PV, so O may be rescaled below. The K stage of tile j goes back to the
+      // producer.
       tc::fence_after_sync();
-      if (warp == 4 * wg && lane == 0) {
-        tc::mbar_arrive(ke0 + 8 * (j % NK));
-        if (!VREL && j >= 2) tc::mbar_arrive(ve0 + 8 * ((j - 2) % NV));  // (with VREL: the MMA thread's commit)
-      }
+      if (warp == 4 * wg && lane == 0) tc::mbar_arrive(ke0 + 8 * (j % NK));
       uint32_t sv[KT];
 #pragma unroll
       for (int q4 = 0; q4 < KT / 32; ++q4)
@@ -747,19 +738,20 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_c
         for (int c = 0; c < KT; ++c)
           if (!((w[c >> 5] >> (c & 31)) & 1u)) sv[c] = 0xff800000u;
       }
-      // row maximum of the raw scores as a tree of three-input maxima (scale
-      // > 0, so it commutes with the scaling)
-      float mt[43];
+      // row maximum of the raw scores (scale > 0, so it commutes with the
+      // scaling): eight running maxima of two scores per step
+      float mt[8];
 #pragma unroll
-      for (int i = 0; i < 42; ++i)
-        mt[i] = max3f(__uint_as_float(sv[3 * i]), __uint_as_float(sv[3 * i + 1]), __uint_as_float(sv[3 * i + 2]));
-      mt[42] = fmaxf(__uint_as_float(sv[126]), __uint_as_float(sv[127]));
+      for (int i = 0; i < 8; ++i)
+        mt[i] = max3f(__uint_as_float(sv[2 * i]), __uint_as_float(sv[2 * i + 1]), __uint_as_float(sv[16 + i]));
 #pragma unroll
-      for (int i = 0; i < 14; ++i) mt[i] = max3f(mt[3 * i], mt[3 * i + 1], mt[3 * i + 2]);
-      mt[14] = mt[42];  // 15 left
+      for (int i = 24; i < 120; i += 16)
 #pragma unroll
-      for (int i = 0; i < 5; ++i) mt[i] = max3f(mt[3 * i], mt[3 * i + 1], mt[3 * i + 2]);
-      const float mx = max3f(max3f(mt[0], mt[1], mt[2]), mt[3], mt[4]) * p.scale_log2;
+        for (int e = 0; e < 8; ++e)
+          mt[e] = max3f(mt[e], __uint_as_float(sv[i + 2 * e]), __uint_as_float(sv[i + 2 * e + 1]));
+#pragma unroll
+      for (int e = 0; e < 8; ++e) mt[e] = fmaxf(mt[e], __uint_as_float(sv[120 + e]));
+      const float mx = max3f(max3f(mt[0], mt[1], mt[2]), max3f(mt[3], mt[4], mt[5]), fmaxf(mt[6], mt[7])) * p.scale_log2;
       const bool resc = mx > m_ref + RESCALE;
       float corr = 1.f;
       if (resc) {
@@ -770,179 +762,83 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_c
         m_ref = mx;
         l *= corr;
       }
-      if constexpr (SPLIT) {
-        // P in two halves of 64 keys: exponents scale * s - m two at a time
-        // (f32x2 FMA), their sum two at a time (f32x2 add), P as bf16 pairs
-        // over the first 64 columns of S, 32 keys per step
-        const float nmu = (m_ref == -INFINITY) ? 0.f : -m_ref;
-        const uint64_t scale2 = f32x2(p.scale_log2, p.scale_log2), nmu2 = f32x2(nmu, nmu);
-        uint64_t acc2[2] = {f32x2(0.f, 0.f), f32x2(0.f, 0.f)};
-        uint64_t wacc2 = f32x2(0.f, 0.f);  // entropy: sum of P e over the tile
-        auto p_step = [&](int q4) {
-          uint32_t pk[16];
+      // P in two parts: exponents scale * s - m two at a time
+      // (f32x2 FMA), their sum two at a time (f32x2 add), P as bf16 pairs
+      // over the first 64 columns of S, 32 keys per step
+      const float nmu = (m_ref == -INFINITY) ? 0.f : -m_ref;
+      const uint64_t scale2 = f32x2(p.scale_log2, p.scale_log2), nmu2 = f32x2(nmu, nmu);
+      uint64_t acc2[2] = {f32x2(0.f, 0.f), f32x2(0.f, 0.f)};
+      uint64_t wacc2 = f32x2(0.f, 0.f);  // entropy: sum of P e over the tile
+      auto p_step = [&](int q4) {
+        uint32_t pk[16];
 #pragma unroll
-          for (int c = 0; c < 16; ++c) {
-            float e0, e1;
-            f32x2_split(ffma2(f32x2(__uint_as_float(sv[32 * q4 + 2 * c]), __uint_as_float(sv[32 * q4 + 2 * c + 1])),
-                              scale2, nmu2),
-                        e0, e1);
-            const float p0 = tc::ex2(e0), p1 = tc::ex2(e1);
-            acc2[c & 1] = fadd2(acc2[c & 1], f32x2(p0, p1));
-            // masked slots have e = -inf and P = 0: clamp e so that P e is 0, not NaN
-            if (ENT) wacc2 = ffma2(f32x2(p0, p1), f32x2(fmaxf(e0, -200.f), fmaxf(e1, -200.f)), wacc2);
-            pk[c] = pack_bf16x2(p0, p1);
-          }
-          tc::tmem_st16(tl + 16 * q4, pk);
-        };
-        p_step(0);
-        p_step(1);
-        // Before the first half goes to the MMA thread (with half the scores
-        // consumed, so that the registers allow it): slots past the sequence
-        // end may hold any bits (0 * NaN = NaN in the PV product), so their V
-        // rows are zeroed once the tile's copy has landed (a later landing
-        // would undo the zeros); and O follows a raised reference before
-        // PV_j's first half adds to it.
-        if (c1 - s0 < KT) {
-          const int st = j % NV;
-          if (!__all_sync(0xffffffffu, tc::mbar_wait(vf0 + 8 * st, (j / NV) & 1, abort_flag, wait_ns))) {
-            give_up();
-            ok = false;
-            break;
-          }
-          const int first = c1 - s0, nz = (KT - first) * NR * 8;
-          for (int i = 32 * (warp & 3) + lane; i < nz; i += 32 * n_act) {
-            const int r = first + i / (NR * 8), rc = i % (NR * 8);
-            const uint32_t dst = v_s(st) + (rc >> 3) * KV_REGION + r * 128 + ((rc & 7) << 4);
-            asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};" ::"r"(dst), "r"(0u) : "memory");
-          }
-          tc::fence_proxy_async_smem();
+        for (int c = 0; c < 16; ++c) {
+          float e0, e1;
+          f32x2_split(ffma2(f32x2(__uint_as_float(sv[32 * q4 + 2 * c]), __uint_as_float(sv[32 * q4 + 2 * c + 1])),
+                            scale2, nmu2),
+                      e0, e1);
+          const float p0 = tc::ex2(e0), p1 = tc::ex2(e1);
+          acc2[c & 1] = fadd2(acc2[c & 1], f32x2(p0, p1));
+          // masked slots have e = -inf and P = 0: clamp e so that P e is 0, not NaN
+          if (ENT) wacc2 = ffma2(f32x2(p0, p1), f32x2(fmaxf(e0, -200.f), fmaxf(e1, -200.f)), wacc2);
+          pk[c] = pack_bf16x2(p0, p1);
         }
-        if (ii > 0 && __any_sync(0xffffffffu, resc)) {
+        tc::tmem_st16(tl + 16 * q4, pk);
+      };
 #pragma unroll
-          for (int c4 = 0; c4 < D / 32; ++c4) {
-            uint32_t ov[32];
-            tc::tmem_ld32(tl + 128 + c4 * 32, ov);
-            tc::tmem_wait_ld();
-#pragma unroll
-            for (int e = 0; e < 32; ++e) ov[e] = __float_as_uint(__uint_as_float(ov[e]) * corr);
-            tc::tmem_st32(tl + 128 + c4 * 32, ov);
-          }
-        }
-        // One thread also waits for the copies the MMA thread needs next, V_j
-        // for the first half of PV_j, then K_{j+2} for QK_{j+2} (usually
-        // landed by now; the waits overlap the TMEM stores): the MMA thread
-        // then waits for P alone.
-        bool kv_ok = true;
-        if (warp == 4 * wg && lane == 0)
-          kv_ok = tc::mbar_wait(vf0 + 8 * (j % NV), (j / NV) & 1, abort_flag, wait_ns);
-        if (!__all_sync(0xffffffffu, kv_ok)) {
+      for (int q4 = 0; q4 < FIRST / 32; ++q4) p_step(q4);
+      // Before the first part goes to the MMA warp (with half the scores
+      // consumed, so that the registers allow it): slots past the sequence
+      // end may hold any bits (0 * NaN = NaN in the PV product), so their V
+      // rows are zeroed once the tile's copy has landed (a later landing
+      // would undo the zeros); and O follows a raised reference before
+      // PV_j's first part adds to it.
+      if (c1 - s0 < KT) {
+        const int st = j % NV;
+        if (!__all_sync(0xffffffffu, tc::mbar_wait(vf0 + 8 * st, (j / NV) & 1, abort_flag, wait_ns))) {
           give_up();
           ok = false;
           break;
         }
-        tc::tmem_wait_st();
-        tc::fence_before_sync();
-        tc::mbar_arrive(bph0 + 8 * wg);
-        p_step(2);
-        p_step(3);
-        {
-          float a0, a1, b0, b1;
-          f32x2_split(acc2[0], a0, a1);
-          f32x2_split(acc2[1], b0, b1);
-          l += (a0 + a1) + (b0 + b1);
-          if (ENT) {
-            f32x2_split(wacc2, a0, a1);
-            wsum += a0 + a1;
-          }
+        const int first = c1 - s0, nz = (KT - first) * NR * 8;
+        for (int i = 32 * (warp & 3) + lane; i < nz; i += 32 * n_act) {
+          const int r = first + i / (NR * 8), rc = i % (NR * 8);
+          const uint32_t dst = v_s(st) + (rc >> 3) * KV_REGION + r * 128 + ((rc & 7) << 4);
+          asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};" ::"r"(dst), "r"(0u) : "memory");
         }
-        if (warp == 4 * wg && lane == 0)
-          kv_ok = j + 2 >= ntiles ||
-                  tc::mbar_wait(kf0 + 8 * ((j + 2) % NK), ((j + 2) / NK) & 1, abort_flag, wait_ns);
-        if (!__all_sync(0xffffffffu, kv_ok)) {
-          give_up();
-          ok = false;
-          break;
-        }
-      } else {
-        const float nmu = (m_ref == -INFINITY) ? 0.f : -m_ref;
-        // exponents scale * s - m two at a time (f32x2 FMA), their sum two at a
-        // time (f32x2 add), P as bf16 pairs
-        const uint64_t scale2 = f32x2(p.scale_log2, p.scale_log2), nmu2 = f32x2(nmu, nmu);
-        uint64_t acc2[2] = {f32x2(0.f, 0.f), f32x2(0.f, 0.f)};
-        uint64_t wacc2 = f32x2(0.f, 0.f);  // entropy: sum of P e over the tile
+        tc::fence_proxy_async_smem();
+      }
+      if (ii > 0 && __any_sync(0xffffffffu, resc)) {
 #pragma unroll
-        for (int q4 = 0; q4 < KT / 32; ++q4) {
-          uint32_t pk[16];
+        for (int c4 = 0; c4 < D / 32; ++c4) {
+          uint32_t ov[32];
+          tc::tmem_ld32(tl + 128 + c4 * 32, ov);
+          tc::tmem_wait_ld();
 #pragma unroll
-          for (int c = 0; c < 16; ++c) {
-            float e0, e1;
-            f32x2_split(ffma2(f32x2(__uint_as_float(sv[32 * q4 + 2 * c]), __uint_as_float(sv[32 * q4 + 2 * c + 1])),
-                              scale2, nmu2),
-                        e0, e1);
-            const float p0 = tc::ex2(e0), p1 = tc::ex2(e1);
-            acc2[c & 1] = fadd2(acc2[c & 1], f32x2(p0, p1));
-            // masked slots have e = -inf and P = 0: clamp e so that P e is 0, not NaN
-            if (ENT) wacc2 = ffma2(f32x2(p0, p1), f32x2(fmaxf(e0, -200.f), fmaxf(e1, -200.f)), wacc2);
-            pk[c] = pack_bf16x2(p0, p1);
-          }
-          tc::tmem_st16(tl + 16 * q4, pk);  // P (bf16 pairs) over the first 64 columns of S
-        }
-        {
-          float a0, a1, b0, b1;
-          f32x2_split(acc2[0], a0, a1);
-          f32x2_split(acc2[1], b0, b1);
-          l += (a0 + a1) + (b0 + b1);
-          if (ENT) {
-            f32x2_split(wacc2, a0, a1);
-            wsum += a0 + a1;
-          }
-        }
-        if (c1 - s0 < KT) {
-          // slots past the sequence end may hold any bits (0 * NaN = NaN in the
-          // PV product): zero those V rows before the MMA reads them, once the
-          // tile's copy has landed (a later landing would undo the zeros)
-          const int st = j % NV;
-          if (!__all_sync(0xffffffffu, tc::mbar_wait(vf0 + 8 * st, (j / NV) & 1, abort_flag, wait_ns))) {
-            give_up();
-            ok = false;
-            break;
-          }
-          const int first = c1 - s0, nz = (KT - first) * NR * 8;
-          for (int i = 32 * (warp & 3) + lane; i < nz; i += 32 * n_act) {
-            const int r = first + i / (NR * 8), rc = i % (NR * 8);
-            const uint32_t dst = v_s(st) + (rc >> 3) * KV_REGION + r * 128 + ((rc & 7) << 4);
-            asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};" ::"r"(dst), "r"(0u) : "memory");
-          }
-          tc::fence_proxy_async_smem();
-        }
-        if (ii > 0 && __any_sync(0xffffffffu, resc)) {
-#pragma unroll
-          for (int c4 = 0; c4 < D / 32; ++c4) {
-            uint32_t ov[32];
-            tc::tmem_ld32(tl + 128 + c4 * 32, ov);
-            tc::tmem_wait_ld();
-#pragma unroll
-            for (int e = 0; e < 32; ++e) ov[e] = __float_as_uint(__uint_as_float(ov[e]) * corr);
-            tc::tmem_st32(tl + 128 + c4 * 32, ov);
-          }
-        }
-        // One thread also waits for the copies the MMA thread needs next, V_j
-        // and K_{j+2} (usually landed by now; the wait overlaps the TMEM
-        // stores): the MMA thread then waits for P_j alone.
-        bool kv_ok = true;
-        if (warp == 4 * wg && lane == 0)
-          kv_ok = tc::mbar_wait(vf0 + 8 * (j % NV), (j / NV) & 1, abort_flag, wait_ns) &&
-                  (j + 2 >= ntiles ||
-                   tc::mbar_wait(kf0 + 8 * ((j + 2) % NK), ((j + 2) / NK) & 1, abort_flag, wait_ns));
-        if (!__all_sync(0xffffffffu, kv_ok)) {
-          give_up();
-          ok = false;
-          break;
+          for (int e = 0; e < 32; ++e) ov[e] = __float_as_uint(__uint_as_float(ov[e]) * corr);
+          tc::tmem_st32(tl + 128 + c4 * 32, ov);
         }
       }
       tc::tmem_wait_st();
       tc::fence_before_sync();
-      tc::mbar_arrive(bp0 + 8 * wg);
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(bph0 + 8 * wg);
+#pragma unroll
+      for (int q4 = FIRST / 32; q4 < KT / 32; ++q4) p_step(q4);
+      {
+        float a0, a1, b0, b1;
+        f32x2_split(acc2[0], a0, a1);
+        f32x2_split(acc2[1], b0, b1);
+        l += (a0 + a1) + (b0 + b1);
+        if (ENT) {
+          f32x2_split(wacc2, a0, a1);
+          wsum += a0 + a1;
+        }
+      }
+      tc::tmem_wait_st();
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(bp0 + 8 * wg);
     }
     // all MMAs done (the issuer commits this single-use barrier after its last PV)
     if (ok && nw > 0 && !__all_sync(0xffffffffu, tc::mbar_wait(bdrain, 0, abort_flag, wait_ns))) {
@@ -1286,12 +1182,8 @@ template <int D, bool ENT>
 dreams_status_t launch(const AttnParams &a, const AttnPlan &pl, const dreams_kv_cache_t *kv, const void *k,
                        const void *v, int B, int64_t q_stride_b, int64_t q_stride_t, cudaStream_t stream) {
   constexpr size_t smem = smem_bytes<D>();
-  void (*kernel)(const TcParams) =
-      a.mode == ATTN_CAUSAL ? tree_attn_tc_kernel<D, ENT, false, false>
-                            : (kv->page_table != nullptr ? tree_attn_tc_kernel<D, ENT, true, true>
-                                                         : tree_attn_tc_kernel<D, ENT, true, false>);
   {
-    const dreams_status_t st = ensure_max_dynamic_smem(reinterpret_cast<const void *>(kernel), int(smem));
+    const dreams_status_t st = ensure_max_dynamic_smem(reinterpret_cast<const void *>(tree_attn_tc_kernel<D, ENT>), int(smem));
     if (st != DREAMS_OK) return st;
   }
   TcParams P;
@@ -1308,7 +1200,7 @@ dreams_status_t launch(const AttnParams &a, const AttnPlan &pl, const dreams_kv_
     if (st != DREAMS_OK) return st;
   }
   const int64_t ctas = int64_t(B) * pl.nsplit * a.Hkv * pl.nrb;
-  const dreams_status_t st = launch_kernel(kernel, dim3(unsigned(ctas)), dim3(THREADS), smem, stream, P);
+  const dreams_status_t st = launch_kernel(tree_attn_tc_kernel<D, ENT>, dim3(unsigned(ctas)), dim3(THREADS), smem, stream, P);
   if (st != DREAMS_OK || pl.nsplit == 1) return st;
   const int64_t rows = int64_t(B) * a.Hkv * pl.nrb * ROWS;
   return launch_kernel(tree_attn_merge_kernel<D, ENT>, dim3(unsigned((rows + 7) / 8)), dim3(256), 0, stream, a);
