@@ -974,8 +974,6 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_c
 // once that grid has completed and its writes are visible.
 template <int D, bool ENT>
 __global__ void __launch_bounds__(256) tree_attn_merge_kernel(const AttnParams p) {
-  grid_wait();
-  launch_successor();
   constexpr int NL = D / 4;  // lanes holding 4 columns each
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t row = int64_t(blockIdx.x) * 8 + warp;
@@ -985,20 +983,32 @@ __global__ void __launch_bounds__(256) tree_attn_merge_kernel(const AttnParams p
   const int64_t bg = item / p.nrb;
   const int g = int(bg % p.Hkv);
   const int b = int(bg / p.Hkv);
-  if (b >= p.B) return;
-  const int T = __ldg(p.tree_len + b);
-  const int L = __ldg(p.kv_len + b);
+  // What the row is, from the call's inputs, while the attention grid runs;
+  // then the wait, on every path: a grid that did not wait could complete
+  // before the one ahead of it.
+  const bool seq = b < p.B;
+  const int T = seq ? __ldcg(p.tree_len + b) : 0;
+  const int L = seq ? __ldcg(p.kv_len + b) : 0;
+  int bad = 0;  // the attention kernel skipped malformed trees; so does the merge
+  if (p.mode == ATTN_TREE && seq) {
+    for (int i = lane; i < ::min(T, p.T_max); i += 32) {
+      const int par = __ldcg(p.parent + int64_t(b) * p.T_max + i);
+      bad |= (i == 0) ? (par != -1) : (par < 0 || par >= i);
+    }
+  }
   const int total = key_total(p, L, T);
-  if (T < 1 || T > p.T_max || L < 0 || total > p.capacity || total < 1) return;
   const int t0 = rb * p.TB;
-  if (t0 >= T || r >= ::min(p.TB, T - t0) * p.G) return;
   // splits of the row block (it was written directly when there is one) and
   // of this row (a causal row's keys end at its own slot)
   const int kend = p.mode == ATTN_CAUSAL ? L + ::min(T, t0 + p.TB) : total;
   const int nsplit_blk = (kend + p.chunk - 1) / p.chunk;
-  if (nsplit_blk == 1) return;
   const int tn = r / p.G;
   const int nsplit_b = p.mode == ATTN_CAUSAL ? (L + t0 + tn + 1 + p.chunk - 1) / p.chunk : nsplit_blk;
+  const bool live = T >= 1 && T <= p.T_max && L >= 0 && total <= p.capacity && total >= 1 && t0 < T &&
+                    r < ::min(p.TB, T - t0) * p.G && nsplit_blk > 1;
+  grid_wait();
+  launch_successor();
+  if (!live) return;
 
   const int64_t sbase = item * p.nsplit * ROWS + r;
   float4 x[8];
@@ -1009,13 +1019,6 @@ __global__ void __launch_bounds__(256) tree_attn_merge_kernel(const AttnParams p
                : make_float4(0.f, 0.f, 0.f, 0.f);
   const float2 ml = lane < nsplit_b ? __ldcg(p.ws_ml + sbase + int64_t(lane) * ROWS) : make_float2(-INFINITY, 0.f);
   const float wl = (ENT && lane < nsplit_b) ? __ldcg(p.ws_w + sbase + int64_t(lane) * ROWS) : 0.f;
-  int bad = 0;  // the attention kernel skipped malformed trees; so does the merge
-  if (p.mode == ATTN_TREE) {
-    for (int i = lane; i < T; i += 32) {
-      const int par = __ldg(p.parent + int64_t(b) * p.T_max + i);
-      bad |= (i == 0) ? (par != -1) : (par < 0 || par >= i);
-    }
-  }
   // a split that gave up waiting left a negative sum: the row stays untouched
   bad |= ml.y < 0.f;
   if (__any_sync(0xffffffffu, bad)) return;
