@@ -97,7 +97,6 @@ __device__ __forceinline__ void add_words(const uint4 *w, float (&acc)[8]) {
 template <typename T>
 __global__ void __launch_bounds__(MAX_PART_THREADS) importance_partial_kernel(const ImpParams p) {
   grid_wait();
-  launch_successor();
   constexpr int WPG = int(sizeof(T)) / 2;  // words per 8-column group
   constexpr int U = 8 / WPG;               // rows in flight
   const int b = blockIdx.z, c = blockIdx.y;
