@@ -34,6 +34,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "tc.cuh"
 
 namespace dreams {
 namespace {
@@ -1139,11 +1140,13 @@ __global__ void __launch_bounds__(TAIL_THREADS) verify_tail_kernel(const StepPar
 // visited, as exponentials in shared memory (each thread's relative to its own
 // maximum m, with the factor a = 2^((m - M) k2) to the row's maximum M kept in
 // a register). Only the rows of visited nodes are read. A sum over the
-// vocabulary: warps reduce their threads' values, warp 0 the warps' and stores
-// the CTA's value into every CTA's shared memory (distributed shared memory),
-// one cluster barrier, then each warp combines the cs values in rank order:
-// all CTAs hold bit-identical results, take the same decisions and pass the
-// same cluster barriers. The rows' maxima and exponential sums take one such
+// vocabulary: warps reduce their threads' values, warp 0 the warps' and sends
+// the CTA's value into every CTA's shared memory (distributed shared memory;
+// asynchronous stores that complete on the receiving CTA's barrier), then each
+// warp combines the cs values in rank order: all CTAs hold bit-identical
+// results, take the same decisions and make the same exchanges. The walk is a
+// chain of such exchanges, so their latency is its time: one store's flight
+// instead of a cluster barrier's arrival and release. The rows' maxima and exponential sums take one such
 // exchange of (maximum, sum) pairs.
 constexpr int SPEC_THREADS = 512;                    // 16 warps
 constexpr int SPEC_CHUNK = 8 * SPEC_THREADS;         // values per chunk: 8 per thread
@@ -1183,17 +1186,18 @@ __device__ __forceinline__ uint32_t cluster_addr(const void *local_ptr, uint32_t
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
   return ra;
 }
-__device__ __forceinline__ void st_cluster_f4(const float4 *local_ptr, uint32_t rank, float4 v) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr(local_ptr, rank)), "f"(v.x),
-               "f"(v.y), "f"(v.z), "f"(v.w)
-               : "memory");
+// Stores v at local_ptr of CTA `rank`; its 16 bytes count on that CTA's barrier `bar`.
+__device__ __forceinline__ void st_async_f4(const float4 *local_ptr, const uint64_t *bar, uint32_t rank, float4 v) {
+  asm volatile(
+      "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
+          cluster_addr(local_ptr, rank)),
+      "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(cluster_addr(bar, rank))
+      : "memory");
 }
-__device__ __forceinline__ void st_cluster_s32(const int32_t *local_ptr, uint32_t rank, int32_t v) {
-  asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(cluster_addr(local_ptr, rank)), "r"(v) : "memory");
-}
-
 struct SpecShared {
   float4 slot[2][SPEC_MAX_CS];       // [parity][rank]: every CTA's partial of the current exchange
+  uint64_t bar[2];                   // [parity]: the exchange's cs partials have arrived
+  int32_t zero, late;                // (never set; an exchange did not arrive in time)
   float chunk[SPEC_MAX_J][16];       // the bonus draw: per-warp sums of each chunk
   float red[16];                     // the bonus draw: per-warp sums of the slice
   float4 red4[16];                   // per-warp partials of a sum or of (maximum, sum) pairs
@@ -1203,7 +1207,7 @@ struct SpecShared {
   float cxt[64], cxd[64];  // the target / draft logits at each child's draft token
   float cu[64];            // u_acc of each child
   int32_t pick;            // the draw inside this CTA's slice
-  int32_t bonus;           // rank 0: the bonus token, written by the CTA that drew it
+  int32_t pg[2];           // page-table entries of the tree's slots
   int32_t cmd;
 };
 
@@ -1238,50 +1242,66 @@ __device__ __forceinline__ float warp_sum_bcast(float v) {
   return __shfl_sync(0xffffffffu, v, 0);  // lane 0's bits on every lane
 }
 
+// The maximum over the warp's lanes (a NaN loses), on every lane.
+__device__ __forceinline__ float warp_max(float v) {
+  float m;
+  asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(v));
+  return m;
+}
+
 // (maximum, sum of 2^((x - maximum) k2)) of two rows over the warp's lanes,
 // from each lane's pair (x, y) and (z, w); lane 0's bits on every lane.
 __device__ __forceinline__ float4 ms4_lanes(float4 v, float k2) {
-  float Mt = v.x, Md = v.z;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    Mt = fmaxf(Mt, __shfl_xor_sync(0xffffffffu, Mt, off));
-    Md = fmaxf(Md, __shfl_xor_sync(0xffffffffu, Md, off));
-  }
+  const float Mt = warp_max(v.x), Md = warp_max(v.z);
   const float st = v.x == -INFINITY ? 0.f : v.y * exp2f_approx((v.x - Mt) * k2);
   const float sd = v.z == -INFINITY ? 0.f : v.w * exp2f_approx((v.z - Md) * k2);
   return make_float4(Mt, warp_sum_bcast(st), Md, warp_sum_bcast(sd));
 }
 
-// A sum over the cluster: warps, then warp 0 over the warps, then one value
-// per CTA into slot [parity][rank] of every CTA; after the cluster barrier
-// every warp combines the cs values in lane order (the same bits everywhere).
-__device__ __forceinline__ float spec_cluster_sum(SpecShared &sh, float v, int parity, int cs, uint32_t rank) {
+// One exchange of the cluster, number x (0, 1, ...): warp 0's lane r sends this
+// CTA's partial to CTA r, and every thread waits for the cs partials sent to
+// its own CTA. Exchanges alternate between two sets of slots and barriers: a
+// CTA sends number x + 2 only once it holds every partial of x + 1, and those
+// were sent after their senders' threads had read the slots of x.
+__device__ __forceinline__ void spec_send(SpecShared &sh, float4 cta, int x, int cs, uint32_t rank) {
+  const int lane = threadIdx.x & 31;
+  if (lane == 0) tc::mbar_arrive_expect_tx(smem_u32(&sh.bar[x & 1]), uint32_t(cs) * 16u);
+  if (lane < cs) st_async_f4(&sh.slot[x & 1][rank], &sh.bar[x & 1], uint32_t(lane), cta);
+}
+__device__ __forceinline__ void spec_arrived(SpecShared &sh, int x) {
+  const uint32_t bar = smem_u32(&sh.bar[x & 1]);
+  if (!tc::mbar_wait_cluster(bar, (x >> 1) & 1, &sh.zero)) sh.late = 1;  // (after 2 s: flagged at the end)
+}
+
+// A sum over the cluster: warps, then warp 0 over the warps, then the CTAs'
+// values, combined in rank order on every warp (the same bits everywhere).
+__device__ __forceinline__ float spec_cluster_sum(SpecShared &sh, float v, int x, int cs, uint32_t rank) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float wv = warp_sum_bcast(v);
-  if (lane == 0) sh.red4[warp] = make_float4(wv, 0.f, 0.f, 0.f);
+  if (lane == 0) sh.red[warp] = wv;
   __syncthreads();
   if (warp == 0) {
-    const float cta = warp_sum_bcast(lane < 16 ? sh.red4[lane].x : 0.f);
-    if (lane < cs) st_cluster_f4(&sh.slot[parity][rank], uint32_t(lane), make_float4(cta, 0.f, 0.f, 0.f));
+    const float cta = warp_sum_bcast(lane < 16 ? sh.red[lane] : 0.f);
+    spec_send(sh, make_float4(cta, 0.f, 0.f, 0.f), x, cs, rank);
   }
-  cluster_sync();
-  return warp_sum_bcast(lane < cs ? sh.slot[parity][lane].x : 0.f);
+  spec_arrived(sh, x);
+  return warp_sum_bcast(lane < cs ? sh.slot[x & 1][lane].x : 0.f);
 }
 
 // The rows' maxima and exponential sums over the cluster from each thread's
 // (m_t, s_t, m_d, s_d), s = sum 2^((x - m) k2): (Mt, Zt, Md, Zd). The same
 // three levels as a sum: warps, warp 0 over the warps, the CTAs.
-__device__ float4 spec_cluster_ms(SpecShared &sh, float4 v, int parity, int cs, uint32_t rank, float k2) {
+__device__ float4 spec_cluster_ms(SpecShared &sh, float4 v, int x, int cs, uint32_t rank, float k2) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float4 w = ms4_lanes(v, k2);
   if (lane == 0) sh.red4[warp] = w;
   __syncthreads();
   if (warp == 0) {
     const float4 cta = ms4_lanes(lane < 16 ? sh.red4[lane] : make_float4(-INFINITY, 0.f, -INFINITY, 0.f), k2);
-    if (lane < cs) st_cluster_f4(&sh.slot[parity][rank], uint32_t(lane), cta);
+    spec_send(sh, cta, x, cs, rank);
   }
-  cluster_sync();
-  return ms4_lanes(lane < cs ? sh.slot[parity][lane] : make_float4(-INFINITY, 0.f, -INFINITY, 0.f), k2);
+  spec_arrived(sh, x);
+  return ms4_lanes(lane < cs ? sh.slot[x & 1][lane] : make_float4(-INFINITY, 0.f, -INFINITY, 0.f), k2);
 }
 
 // Warp 0: the parent and token rows of a sequence into sh (entries past
@@ -1304,90 +1324,61 @@ __device__ int spec_tree_warp(SpecShared &sh, const int (&pre_par)[2], const int
   return __any_sync(0xffffffffu, bad) ? DREAMS_DATA_BAD_PARENT : 0;
 }
 
-// This thread's values of one slice as floats into e (values past V: -inf);
-// returns their maximum.
+// Where a thread's 8 values of chunk j sit in a slice: two float4 half a chunk
+// apart, so that a warp's accesses cover whole 128-byte rows (side by side the
+// two would conflict on every access).
+__device__ __forceinline__ int spec_at(int j, int half) {
+  return j * SPEC_CHUNK + half * (SPEC_CHUNK / 2) + 4 * int(threadIdx.x);
+}
+
+// This thread's raw words of one slice of a row (values past V: -inf).
 template <typename T>
-__device__ __forceinline__ float spec_store_raw(const SpecParams &p, const uint4 (&w)[SPEC_MAX_J][sizeof(T) / 2],
-                                                float *e) {
+__device__ __forceinline__ void spec_issue(const SpecParams &p, const T *row, int64_t v0,
+                                           uint4 (&w)[SPEC_MAX_J][sizeof(T) / 2]) {
+  const int warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int j = 0; j < SPEC_MAX_J; ++j)
+    if (j < p.J) sub_words<T>(row + v0, p.V - v0, p.vec_ok, int64_t(j) * (SPEC_CHUNK / SUB) + warp, w[j]);
+}
+
+// Their exponentials relative to the thread's own maximum into e; returns the
+// maximum and the exponentials' sum. The values go from registers straight to
+// their exponentials: with the raw values staged in shared memory and
+// conflicting accesses a node of the walk (two rows' slices of 16384 bf16)
+// took 11.2 k clk, 8.3 k of them here; now 7.3 k and 4.5 k, most of it the
+// rows' latency from memory.
+template <typename T>
+__device__ __forceinline__ float2 spec_exps(const SpecParams &p, const uint4 (&w)[SPEC_MAX_J][sizeof(T) / 2], float *e) {
   constexpr int NW = int(sizeof(T)) / 2;  // 16-byte words per 8 values
-  const int tid = threadIdx.x;
+  auto value = [&](int j, int i) {
+    return __uint_as_float(Elem<T>::lane_bits(w[j][NW == 1 ? 0 : i >> 2], NW == 1 ? i : (i & 3)));
+  };
   float m = -INFINITY;
 #pragma unroll
   for (int j = 0; j < SPEC_MAX_J; ++j)
     if (j < p.J) {
-      float y[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        y[i] = __uint_as_float(Elem<T>::lane_bits(w[j][NW == 1 ? 0 : i >> 2], NW == 1 ? i : (i & 3)));
-        m = fmaxf(m, y[i]);
-      }
-      float4 *dst = reinterpret_cast<float4 *>(e + j * SPEC_CHUNK + 8 * tid);
-      dst[0] = make_float4(y[0], y[1], y[2], y[3]);
-      dst[1] = make_float4(y[4], y[5], y[6], y[7]);
+      for (int i = 0; i < 8; ++i) m = fmaxf(m, value(j, i));
     }
-  return m;
-}
-
-// This CTA's slices of the target row (and of the draft row when `both`) as
-// floats into et / ed; this thread's maxima of each. bf16 rows have both
-// rows' loads in flight at once; f32 rows are taken one after the other.
-template <typename T>
-__device__ float2 spec_load_rows(const SpecParams &p, const T *trow, const T *drow, bool both, int64_t v0, float *et,
-                                 float *ed) {
-  constexpr int NW = int(sizeof(T)) / 2;
-  const int warp = threadIdx.x >> 5;
-  const int64_t Vs = p.V - v0;  // values of the row from the slice start on
-  float2 m = make_float2(-INFINITY, -INFINITY);
-  uint4 wt[SPEC_MAX_J][NW];
+  float s0 = 0.f, s1 = 0.f;
 #pragma unroll
   for (int j = 0; j < SPEC_MAX_J; ++j)
-    if (j < p.J) sub_words<T>(trow + v0, Vs, p.vec_ok, int64_t(j) * (SPEC_CHUNK / SUB) + warp, wt[j]);
-  if (NW == 1) {
-    uint4 wd[SPEC_MAX_J][NW];
+    if (j < p.J) {
 #pragma unroll
-    for (int j = 0; j < SPEC_MAX_J; ++j)
-      if (both && j < p.J) sub_words<T>(drow + v0, Vs, p.vec_ok, int64_t(j) * (SPEC_CHUNK / SUB) + warp, wd[j]);
-    m.x = spec_store_raw<T>(p, wt, et);
-    if (both) m.y = spec_store_raw<T>(p, wd, ed);
-  } else {
-    m.x = spec_store_raw<T>(p, wt, et);
-    if (both) {
-#pragma unroll
-      for (int j = 0; j < SPEC_MAX_J; ++j)
-        if (j < p.J) sub_words<T>(drow + v0, Vs, p.vec_ok, int64_t(j) * (SPEC_CHUNK / SUB) + warp, wt[j]);
-      m.y = spec_store_raw<T>(p, wt, ed);
+      for (int h = 0; h < 2; ++h) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);  // (every value past V)
+        if (m != -INFINITY) {
+          v.x = exp2f_approx((value(j, 4 * h) - m) * p.k2);
+          v.y = exp2f_approx((value(j, 4 * h + 1) - m) * p.k2);
+          v.z = exp2f_approx((value(j, 4 * h + 2) - m) * p.k2);
+          v.w = exp2f_approx((value(j, 4 * h + 3) - m) * p.k2);
+        }
+        *reinterpret_cast<float4 *>(e + spec_at(j, h)) = v;
+        s0 += v.x + v.y;
+        s1 += v.z + v.w;
+      }
     }
-  }
-  return m;
-}
-
-// e <- 2^((e - M) k2) in place over this thread's values; returns their sum.
-// M = -inf (every value past V): zeros.
-__device__ __forceinline__ float spec_exp_inplace(float *e, float M, float k2, int J) {
-  const int tid = threadIdx.x;
-  if (M == -INFINITY) {
-    for (int j = 0; j < J; ++j) {
-      float4 *q = reinterpret_cast<float4 *>(e + j * SPEC_CHUNK + 8 * tid);
-      q[0] = q[1] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    return 0.f;
-  }
-  float s0 = 0.f, s1 = 0.f;
-  for (int j = 0; j < J; ++j) {
-    float4 *q = reinterpret_cast<float4 *>(e + j * SPEC_CHUNK + 8 * tid);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      float4 v = q[h];
-      v.x = exp2f_approx((v.x - M) * k2);
-      v.y = exp2f_approx((v.y - M) * k2);
-      v.z = exp2f_approx((v.z - M) * k2);
-      v.w = exp2f_approx((v.w - M) * k2);
-      q[h] = v;
-      s0 += v.x + v.y;
-      s1 += v.z + v.w;
-    }
-  }
-  return s0 + s1;
+  return make_float2(m, s0 + s1);
 }
 
 // The residual's numerator at one vocabulary entry: max(0, et - c ed).
@@ -1406,14 +1397,12 @@ __device__ __forceinline__ float spec_weights(const float *et, const float *ed, 
     wj[j] = 0.f;
     if (j < J) {
       const int e0 = j * SPEC_CHUNK + 8 * tid;
-      const float4 *t4 = reinterpret_cast<const float4 *>(et + e0);
-      const float4 *d4 = reinterpret_cast<const float4 *>(ed + e0);
       float w[8];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const float4 tv = t4[h];
+        const float4 tv = *reinterpret_cast<const float4 *>(et + spec_at(j, h));
         if (use_q) {
-          const float4 dv = d4[h];
+          const float4 dv = *reinterpret_cast<const float4 *>(ed + spec_at(j, h));
           w[4 * h] = spec_w(tv.x, dv.x, ct), w[4 * h + 1] = spec_w(tv.y, dv.y, ct);
           w[4 * h + 2] = spec_w(tv.z, dv.z, ct), w[4 * h + 3] = spec_w(tv.w, dv.w, ct);
         } else {
@@ -1504,7 +1493,8 @@ __device__ int spec_slice_draw(SpecShared &sh, const float *et, const float *ed,
     float a = excl;
     int hit = -1, lp = -1;
     for (int i = 0; i < 8; ++i) {
-      const float w = at * (use_q ? spec_w(et[e0 + i], ed[e0 + i], ct) : et[e0 + i]);
+      const int at_i = spec_at(jc, i >> 2) + (i & 3);
+      const float w = at * (use_q ? spec_w(et[at_i], ed[at_i], ct) : et[at_i]);
       a += w;
       if (w > 0.f) lp = e0 + i;
       if (hit < 0 && w > 0.f && a > rem) hit = e0 + i;
@@ -1516,7 +1506,11 @@ __device__ int spec_slice_draw(SpecShared &sh, const float *et, const float *ed,
 }
 
 // One cluster of p.cs CTAs per sequence (grid.x = B * cs): the walk with its
-// decisions, the bonus draw, the outputs and the KV compaction.
+// decisions, the bonus draw, the outputs and the KV compaction. A chain of
+// dependent steps, so its latency is what counts: 16 trees of 32-64 nodes at
+// 128256 bf16 entries took 47.8 us a pass, 32.7 with the root's rows loaded
+// under the tree check, exponentials from registers, conflict-free slices, warp
+// maxima by one instruction, and the outputs written by the CTA that draws.
 template <typename T>
 __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParams p) {
   grid_wait();
@@ -1533,16 +1527,6 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
   const int64_t v0 = int64_t(rank) * S;
   float *et = spec_dyn, *ed = spec_dyn + S;
   const float k2 = p.k2;
-  // the root's rows towards L2 while the tree is checked
-  for (int j = 0; j < J; ++j) {
-    const int64_t e = v0 + int64_t(j) * SPEC_CHUNK + 8 * tid;
-    if (e < p.V) {
-      const char *tp = static_cast<const char *>(p.tgt) + (rb * p.row_stride + e) * int64_t(sizeof(T));
-      const char *dp = static_cast<const char *>(p.drf) + (rb * p.row_stride + e) * int64_t(sizeof(T));
-      asm volatile("prefetch.L2 [%0];" ::"l"(tp));
-      asm volatile("prefetch.L2 [%0];" ::"l"(dp));
-    }
-  }
   // the tree rows go out with the lengths (rows of T_max entries exist)
   int pre_par[2] = {-1, -1}, pre_tok[2] = {0, 0};
   if (warp == 0) {
@@ -1555,20 +1539,40 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
       }
     }
   }
-  const int TL = __ldg(p.tr.tree_len + b), L = __ldg(p.tr.kv_len + b);
+  const int TL = ld_issue_now(p.tr.tree_len + b), L = ld_issue_now(p.tr.kv_len + b);
+  // the root's rows (bf16: both; f32: the target's) are on their way while the
+  // tree is checked
+  constexpr bool PAIR = sizeof(T) == 2;  // both rows' words fit in registers
+  uint4 wt[SPEC_MAX_J][sizeof(T) / 2], wd[PAIR ? SPEC_MAX_J : 1][PAIR ? sizeof(T) / 2 : 1];
+  spec_issue<T>(p, static_cast<const T *>(p.tgt) + rb * p.row_stride, v0, wt);
+  if constexpr (PAIR) spec_issue<T>(p, static_cast<const T *>(p.drf) + rb * p.row_stride, v0, wd);
+  if (tid == 0) {
+    tc::mbar_init(smem_u32(&sh.bar[0]), 1);
+    tc::mbar_init(smem_u32(&sh.bar[1]), 1);
+    tc::fence_barrier_init();
+    sh.zero = sh.late = 0;
+  }
   if (warp == 0) {
     int bad = 0;
     if (TL < 1 || TL > Tm) bad = DREAMS_DATA_BAD_TREE_LEN;
     else if (L < 0 || L > p.kv.capacity - TL) bad = DREAMS_DATA_BAD_KV_LEN;
     else bad = spec_tree_warp(sh, pre_par, pre_tok, TL);
+    // the entries of the pages that hold the tree's slots, for the compaction
+    if (lane < 2) {
+      const int pg = (L >> 6) + lane;
+      sh.pg[lane] = !bad && p.kv.page_table != nullptr && pg < p.kv.pages_per_seq
+                        ? __ldg(p.kv.page_table + int64_t(b) * p.kv.pages_per_seq + pg)
+                        : -1;
+    }
     if (lane == 0) {
       sh.cmd = bad;
       if (bad && rank == 0) flag(p.status, bad);
     }
   }
-  __syncthreads();
+  cluster_sync();  // every CTA's barriers are ready for the others' partials
   const bool bad = sh.cmd != 0;
-  int n = -1, bonus = 0, parity = 0;
+  int n = -1, bonus = 0, xc = 0;  // xc: exchanges made
+  int writer = 0;  // the CTA that draws the bonus and writes the outputs
   if (!bad) {
     int cur = 0;
     n = 0;
@@ -1595,16 +1599,28 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
       }
       const float u_bonus = ld_now_f32(p.u_res + rb + cur);
       // the rows' maxima and exponential sums: per thread, then over the cluster
-      const float2 m = spec_load_rows<T>(p, trow, drow, try_kids, v0, et, ed);
+      if (cur != 0) {
+        spec_issue<T>(p, trow, v0, wt);
+        if constexpr (PAIR)
+          if (try_kids) spec_issue<T>(p, drow, v0, wd);
+      }
       if (my_kid) {  // stored after the rows' loads are out
         sh.cxt[tid] = kid_t;
         sh.cxd[tid] = kid_d;
         sh.cu[tid] = kid_u;
       }
-      const float st = spec_exp_inplace(et, m.x, k2, J);
-      const float sd = try_kids ? spec_exp_inplace(ed, m.y, k2, J) : 0.f;
-      const float4 g = spec_cluster_ms(sh, make_float4(m.x, st, m.y, sd), parity, cs, rank, k2);
-      parity ^= 1;
+      const float2 mt = spec_exps<T>(p, wt, et);
+      float2 md = make_float2(-INFINITY, 0.f);
+      if (try_kids) {
+        if constexpr (PAIR) {
+          md = spec_exps<T>(p, wd, ed);
+        } else {
+          spec_issue<T>(p, drow, v0, wt);
+          md = spec_exps<T>(p, wt, ed);
+        }
+      }
+      const float2 m = make_float2(mt.x, md.x);
+      const float4 g = spec_cluster_ms(sh, make_float4(m.x, mt.y, m.y, md.y), xc++, cs, rank, k2);
       const float Mt = g.x, Zd = g.w;
       // this thread's factors to the rows' maxima (its exponentials are
       // relative to its own maxima), and their ratio for the passes
@@ -1627,17 +1643,15 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
         const float c2 = c + Pu / Zd, ct = c2 * rd;
         float acc0 = 0.f, acc1 = 0.f;
         for (int j = 0; j < J && at > 0.f; ++j) {
-          const float4 *t4 = reinterpret_cast<const float4 *>(et + j * SPEC_CHUNK + 8 * tid);
-          const float4 *d4 = reinterpret_cast<const float4 *>(ed + j * SPEC_CHUNK + 8 * tid);
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
-            const float4 tv = t4[h], dv = d4[h];
+            const float4 tv = *reinterpret_cast<const float4 *>(et + spec_at(j, h));
+            const float4 dv = *reinterpret_cast<const float4 *>(ed + spec_at(j, h));
             acc0 += spec_w(tv.x, dv.x, ct) + spec_w(tv.y, dv.y, ct);
             acc1 += spec_w(tv.z, dv.z, ct) + spec_w(tv.w, dv.w, ct);
           }
         }
-        const float Pn = spec_cluster_sum(sh, at * (acc0 + acc1), parity, cs, rank);
-        parity ^= 1;
+        const float Pn = spec_cluster_sum(sh, at * (acc0 + acc1), xc++, cs, rank);
         if (Pn > 0.f) c = c2, Pu = Pn;  // a zero sum (r == q) keeps the residual
       }
       if (next >= 0) {
@@ -1654,21 +1668,20 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
       float wj[SPEC_MAX_J];
       int last;
       const float tot = spec_weights(et, ed, at, ct, use_q, J, wj, last);
-      // the slice's total (warps, then warp 0 over them) to slot [parity][rank]
-      // of every CTA; lane r then holds slice r's total, the same bits on
-      // every warp of every CTA
+      // the slice's total (warps, then warp 0 over them) to every CTA; lane r
+      // then holds slice r's total, the same bits on every warp of every CTA
       {
         const float wt = warp_sum_bcast(tot);
         if (lane == 0) sh.red[warp] = wt;
         __syncthreads();
         if (warp == 0) {
           const float slice = warp_sum_bcast(lane < 16 ? sh.red[lane] : 0.f);
-          if (lane < cs) st_cluster_f4(&sh.slot[parity][rank], uint32_t(lane), make_float4(slice, 0.f, 0.f, 0.f));
+          spec_send(sh, make_float4(slice, 0.f, 0.f, 0.f), xc, cs, rank);
         }
-        cluster_sync();
+        spec_arrived(sh, xc);
       }
-      const float tr = lane < cs ? sh.slot[parity][lane].x : 0.f;
-      parity ^= 1;
+      const float tr = lane < cs ? sh.slot[xc & 1][lane].x : 0.f;
+      ++xc;
       // their running sum across the lanes, then the crossing slice
       float inc = tr;
 #pragma unroll
@@ -1686,21 +1699,21 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
       const float before = __shfl_sync(0xffffffffu, inc - tr, cr >= 0 ? cr : 0);
       const bool tail = cr < 0;
       if (tail) cr = lastpos;
-      if (cr < 0) {  // no positive weight anywhere (rounding): token 0
-        if (rank == 0 && tid == 0) sh.bonus = 0;
-      } else if (int(rank) == cr) {
+      // that slice's CTA draws and writes the outputs; the others go on to the
+      // compaction (no positive weight anywhere, by rounding: token 0)
+      writer = cr >= 0 ? cr : 0;
+      if (int(rank) == cr) {
         const int e = spec_slice_draw(sh, et, ed, at, ct, use_q, wj, last, J, target - before, tail);
-        if (tid == 0) st_cluster_s32(&sh.bonus, 0, e >= 0 ? int32_t(v0 + e) : 0);
+        if (e >= 0) bonus = int(std::min<int64_t>(v0 + e, p.V - 1));
       }
-      cluster_sync();
-      bonus = int(std::min<int64_t>(std::max(sh.bonus, 0), p.V - 1));  // used by rank 0 only
       break;
     }
   }
-  // outputs (rank 0): path, drafts then the bonus, lengths; the compaction is
-  // shared by the cluster's CTAs
+  // outputs: path, drafts then the bonus, lengths; the compaction is shared by
+  // the cluster's CTAs. (No CTA leaves early: its last exchange brought it every
+  // partial that was ever sent to it.)
   if (warp == 0) {
-    if (rank == 0) {
+    if (int(rank) == writer) {
       const int mp = p.max_path;
       for (int kk = lane; kk < mp; kk += 32) {
         int pv = -1, ov = -1;
@@ -1716,8 +1729,9 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
         p.new_kv_len[b] = n >= 0 ? L + n + 1 : L;
       }
     }
+    if (lane == 0 && sh.late) flag(p.status, DREAMS_DATA_TIMEOUT);
     bool ok = n > 0;
-    if (ok) ok = move_offsets(p.kv, b, L, n, sh.path, sh.src, sh.dst, rank == 0 ? p.status : nullptr);
+    if (ok) ok = move_offsets(p.kv, b, L, n, sh.path, sh.src, sh.dst, rank == 0 ? p.status : nullptr, sh.pg);
     if (lane == 0) sh.cmd = ok ? n : 0;
   }
   __syncthreads();
