@@ -41,13 +41,14 @@ inline dreams_status_t check_launch() {
 // completed and its writes are visible. Each then lets its own successor start
 // (launch_successor, after the wait, so that at most one grid ahead of a
 // running CTA is unfinished). Between back-to-back calls this takes the launch
-// gap out. The streaming kernels of more than one wave (sampling statistics,
-// importance sums) leave it to their CTAs' exits: successors that took their
-// slots early cost 240 rows of 32003 f32 18.2 against 15.5 us, while the
-// attention's merge launched early takes 1.2 us off 18.7. A kernel that reads
-// global memory before its wait may read only
-// what its own predecessor's inputs were (the walk's tree arrays), and reads
-// it through L2 (__ldcg): L1 may hold older lines until the wait.
+// gap out. The sampling statistics let it start at the end of their work:
+// successors that took their slots early, or came only with the CTAs' exits,
+// cost 240 rows of 32003 f32 18 against 15 us; the importance sums leave it to
+// the exits (103.3 against 105.3 us), while the attention's merge launched
+// early takes 1.2 us off 18.7. A kernel that reads global memory before its
+// wait may read only what its own predecessor's inputs were (the walk's tree
+// arrays), and reads it through L2 (__ldcg): L1 may hold older lines until the
+// wait.
 template <typename... Params, typename... Args>
 dreams_status_t launch_kernel(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                               Args... args) {

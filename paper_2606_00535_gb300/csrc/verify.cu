@@ -286,34 +286,6 @@ struct SampleParams {
   float2 *seg;          // [rows][nseg] (m, s)
 };
 
-// The 8 values of this lane in step j of the row (elements j * SUB + 8 lane +
-// i), as floats; values at or past V read as -inf.
-template <typename T>
-__device__ __forceinline__ void sub_load(const T *row, int64_t V, bool vec_ok, int64_t j, float (&x)[8]) {
-  const int lane = threadIdx.x & 31;
-  const int64_t e0 = j * SUB + 8 * lane;
-  if (vec_ok && e0 + 8 <= V) {
-    if (sizeof(T) == 2) {
-      const uint4 v = __ldcs(reinterpret_cast<const uint4 *>(row + e0));
-      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        x[2 * i] = __uint_as_float(w[i] << 16);
-        x[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-      }
-    } else {
-      const uint4 a = __ldcs(reinterpret_cast<const uint4 *>(row + e0));
-      const uint4 b = __ldcs(reinterpret_cast<const uint4 *>(row + e0) + 1);
-      x[0] = __uint_as_float(a.x), x[1] = __uint_as_float(a.y), x[2] = __uint_as_float(a.z);
-      x[3] = __uint_as_float(a.w), x[4] = __uint_as_float(b.x), x[5] = __uint_as_float(b.y);
-      x[6] = __uint_as_float(b.z), x[7] = __uint_as_float(b.w);
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) x[i] = e0 + i < V ? __uint_as_float(Elem<T>::bits(row, e0 + i)) : -INFINITY;
-  }
-}
-
 // 8 consecutive bf16 values at p, which does not start on 16 bytes, as one raw
 // word: from the two aligned 16-byte words that hold them (both hold wanted
 // values) by a shift that is the same in every lane. Sampling 854 rows of
@@ -364,6 +336,14 @@ __device__ __forceinline__ void sub_words(const T *row, int64_t V, bool vec_ok, 
       for (int q = 0; q < int(sizeof(T)) / 2; ++q) w[q] = make_uint4(b[4 * q], b[4 * q + 1], b[4 * q + 2], b[4 * q + 3]);
     }
   }
+}
+
+// The 8 values of raw words, as floats.
+template <typename T>
+__device__ __forceinline__ void words_values(const uint4 (&w)[sizeof(T) / 2], float (&x)[8]) {
+  constexpr int PER = Elem<T>::VEC;  // values per word
+#pragma unroll
+  for (int i = 0; i < 8; ++i) x[i] = __uint_as_float(Elem<T>::lane_bits(w[i / PER], i % PER));
 }
 
 // Maximum (NaN-propagating) and the sum of 2^((x - m) k) of raw words.
@@ -465,12 +445,19 @@ __device__ int sample_select_warp(const SampleParams &p, const T *row, const flo
   const int lane = threadIdx.x & 31;
   const int nseg = p.nseg;
   const float k2 = p.k2;
-  // ---- pass 1: M, Z, and the first segment whose maximum is NaN / +inf
+  // ---- pass 1: M, Z, and the first segment whose maximum is NaN / +inf. The
+  // first batch of segments (all there are, up to 256 k values) stays in
+  // registers for pass 2.
+  float2 v0[8];
+  seg_batch(seg_row, nseg, 0, v0);
   float m_l = -INFINITY, z_l = 0.f;
   int first_nan = INT_MAX, first_inf = INT_MAX;
   for (int base = 0; base < nseg; base += 256) {
     float2 v[8];
-    seg_batch(seg_row, nseg, base, v);
+    if (base > 0) seg_batch(seg_row, nseg, base, v);
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (base == 0) v[i] = v0[i];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int g = base + 8 * lane + i;
@@ -498,8 +485,10 @@ __device__ int sample_select_warp(const SampleParams &p, const T *row, const flo
     const bool want_nan = first_nan != INT_MAX;
     const int g = want_nan ? first_nan : first_inf;
     for (int k = 0; k < 4; ++k) {
+      uint4 w[sizeof(T) / 2];
       float x[8];
-      sub_load<T>(row, p.V, false, 4 * int64_t(g) + k, x);
+      sub_words<T>(row, p.V, p.vec_ok, 4 * int64_t(g) + k, w);
+      words_values<T>(w, x);
       int hit = 8;
 #pragma unroll
       for (int i = 7; i >= 0; --i)
@@ -529,7 +518,10 @@ __device__ int sample_select_warp(const SampleParams &p, const T *row, const flo
   float carry = 0.f;
   for (int base = 0; base < nseg && gs < 0; base += 256) {
     float2 v[8];
-    seg_batch(seg_row, nseg, base, v);
+    if (base > 0) seg_batch(seg_row, nseg, base, v);
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (base == 0) v[i] = v0[i];
     float c[8], ls = 0.f;
     int llast = -1;
 #pragma unroll
@@ -590,13 +582,18 @@ __device__ int sample_select_warp(const SampleParams &p, const T *row, const flo
   }
   if (gs < 0) gs = last;  // t >= every running sum (u = 1, or rounding)
   if (gs < 0) return 0;
-  // ---- the crossing segment again, step by step in index order, in its own scale
+  // ---- the crossing segment again, in index order and its own scale: its four
+  // steps are loaded together (one memory latency instead of up to four)
+  uint4 sw[4][sizeof(T) / 2];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) sub_words<T>(row, p.V, p.vec_ok, 4 * int64_t(gs) + k, sw[k]);
   const float m = __ldcg(seg_row + gs).x;
   float acc = 0.f;
   int last_i = -1;  // last value of positive weight seen (index)
+#pragma unroll
   for (int k = 0; k < 4; ++k) {
     float x[8];
-    sub_load<T>(row, p.V, p.vec_ok, 4 * int64_t(gs) + k, x);
+    words_values<T>(sw[k], x);
     float w[8], ls = 0.f;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -650,18 +647,19 @@ __global__ void __launch_bounds__(SAMPLE_THREADS, sizeof(T) == 2 ? 6 : 4) vocab_
   const int c = blockIdx.x % p.ncta_row;
   const int64_t g0 = int64_t(c) * p.seg_per_cta, g1 = std::min<int64_t>(p.nseg, g0 + p.seg_per_cta);
   sample_stats<T>(p, static_cast<const T *>(p.logits) + r * p.row_stride, p.seg + r * p.nseg, g0, g1);
+  launch_successor();
 }
 
 // Stage 2, one warp per row, chained to stage 1 by programmatic dependent
 // launch (it waits until stage 1 has completed).
 template <typename T>
 __global__ void __launch_bounds__(256) vocab_sample_select_kernel(const SampleParams p, int64_t rows, int32_t *out) {
+  const int64_t r = int64_t(blockIdx.x) * 8 + (threadIdx.x >> 5);
+  const float u = r < rows ? __ldcg(p.u + r) : 0.f;
   grid_wait();
   launch_successor();
-  const int64_t r = int64_t(blockIdx.x) * 8 + (threadIdx.x >> 5);
   if (r >= rows) return;
-  const int idx = sample_select_warp<T>(p, static_cast<const T *>(p.logits) + r * p.row_stride, p.seg + r * p.nseg,
-                                        __ldg(p.u + r));
+  const int idx = sample_select_warp<T>(p, static_cast<const T *>(p.logits) + r * p.row_stride, p.seg + r * p.nseg, u);
   if ((threadIdx.x & 31) == 0) out[r] = idx;
 }
 
@@ -1022,20 +1020,21 @@ __global__ void __launch_bounds__(SAMPLE_THREADS, sizeof(T) == 2 ? 6 : 4) verify
     sample_stats<T>(p.sp, static_cast<const T *>(p.sp.logits) + r * p.sp.row_stride, p.sp.seg + r * p.sp.nseg,
                     g0, g1);
   }
+  launch_successor();
 }
 
 template <typename T>
 __global__ void __launch_bounds__(256) verify_sample_select_kernel(const StepParams p) {
-  grid_wait();
-  launch_successor();
   const int rowg = blockIdx.x * 8 + (threadIdx.x >> 5);
   const int b = rowg / p.tr.T_max, i = rowg % p.tr.T_max;
-  if (b >= p.tr.B) return;
-  const int tl = __ldg(p.tr.tree_len + b);
-  if (tl < 1 || tl > p.tr.T_max || i >= tl) return;
   const int64_t r = int64_t(b) * p.tr.T_max + i;
+  const int tl = b < p.tr.B ? __ldcg(p.tr.tree_len + b) : 0;
+  const float u = b < p.tr.B ? __ldcg(p.sp.u + r) : 0.f;
+  grid_wait();
+  launch_successor();
+  if (b >= p.tr.B || tl < 1 || tl > p.tr.T_max || i >= tl) return;
   const int idx = sample_select_warp<T>(p.sp, static_cast<const T *>(p.sp.logits) + r * p.sp.row_stride,
-                                        p.sp.seg + r * p.sp.nseg, __ldg(p.sp.u + r));
+                                        p.sp.seg + r * p.sp.nseg, u);
   if ((threadIdx.x & 31) == 0) p.pred[r] = idx;
 }
 
