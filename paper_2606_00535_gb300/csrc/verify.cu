@@ -1340,6 +1340,17 @@ __device__ __forceinline__ void spec_issue(const SpecParams &p, const T *row, in
     if (j < p.J) sub_words<T>(row + v0, p.V - v0, p.vec_ok, int64_t(j) * (SPEC_CHUNK / SUB) + warp, w[j]);
 }
 
+// This CTA's slices of a node's two rows towards L2: one lane per 128 bytes.
+template <typename T>
+__device__ __forceinline__ void spec_prefetch(const SpecParams &p, int64_t row, int64_t v0) {
+  constexpr int PER = 128 / int(sizeof(T));  // values per line
+  for (int64_t e = v0 + int64_t(threadIdx.x) * PER; e < std::min<int64_t>(p.V, v0 + int64_t(p.J) * SPEC_CHUNK);
+       e += int64_t(SPEC_THREADS) * PER) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const T *>(p.tgt) + row * p.row_stride + e));
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const T *>(p.drf) + row * p.row_stride + e));
+  }
+}
+
 // Their exponentials relative to the thread's own maximum into e; returns the
 // maximum and the exponentials' sum. The values go from registers straight to
 // their exponentials: with the raw values staged in shared memory and
@@ -1608,6 +1619,9 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
         sh.cxd[tid] = kid_d;
         sh.cu[tid] = kid_u;
       }
+      // the first child is tried first: its rows come towards L2 meanwhile (33.9
+      // -> 33.0 us on the workload below; the first two children's 34.0, all 36.5)
+      if (try_kids) spec_prefetch<T>(p, rb + __ffsll(static_cast<long long>(kids)) - 1, v0);
       const float2 mt = spec_exps<T>(p, wt, et);
       float2 md = make_float2(-INFINITY, 0.f);
       if (try_kids) {
