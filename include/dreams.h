@@ -360,8 +360,9 @@ dreams_status_t dreams_verify_step_speculative(const void *target_logits, const 
  * both pointers 16-byte aligned. The products of bf16 values are exact in
  * f32; the f32 sums run in the tensor cores' order, so a row whose two largest
  * logits lie within rounding of each other may get either index. Two launches:
- * a persistent tcgen05 GEMM (128 x 256 tiles, the argmax of each tile merged
- * into a 64-bit slot per row with atomicMax), then a small kernel that writes
+ * a persistent tcgen05 GEMM on pairs of CTAs (tiles of 256 vocabulary entries by
+ * up to 256 rows, the argmax of each tile merged into a 64-bit slot per row with
+ * atomicMax), then a small kernel that writes
  * the indices and resets the slots. The workspace holds the slots: zero-fill
  * it once when it is allocated; every call leaves it zero-filled. A wait that
  * times out inside the GEMM flags DREAMS_DATA_TIMEOUT in status_word (may be

@@ -216,6 +216,50 @@ __device__ __forceinline__ void mma_commit(uint32_t bar, uint32_t leader) {
       : "memory");
 }
 
+// CTA pairs (cta_group::2): one MMA over the shared memory and the TMEM of the
+// two CTAs of a cluster. A's and D's first half of rows are in the even CTA,
+// the second half in the odd one; each holds half of B's rows. The even CTA
+// issues. Both CTAs allocate and free.
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t dst_smem, uint32_t ncols) {
+  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_relinquish_pair() {
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+// A load into this CTA's shared memory that completes on a barrier of either
+// CTA of the pair (bar: an address of the cluster's window).
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const void *tmap, uint32_t bar, int c0, int c1) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, "
+      "%4}], [%2];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(c0), "r"(c1)
+      : "memory");
+}
+__device__ __forceinline__ void mma_ss_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                            uint32_t accumulate, uint32_t leader) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(leader)
+      : "memory");
+}
+// One arrival on the barrier at this offset in each CTA of the mask.
+__device__ __forceinline__ void mma_commit_pair(uint32_t bar, uint32_t mask, uint32_t leader) {
+  asm volatile(
+      "{\n .reg .pred q;\n .reg .b16 m;\n setp.ne.b32 q, %2, 0;\n cvt.u16.u32 m, %1;\n"
+      " @q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], m;\n}\n" ::"r"(bar),
+      "r"(mask), "r"(leader)
+      : "memory");
+}
+// An arrival on a barrier of any CTA of the cluster (an address of its window).
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
 // Shared-memory matrix descriptor, 128-byte swizzle, sm_100 format:
 // start address >> 4 (bits 0-13), leading-dimension byte offset >> 4
 // (16-29), stride-dimension byte offset >> 4 (32-45), fixed 0b001 (46-48),

@@ -1166,25 +1166,6 @@ struct SpecParams {
   int32_t *status;
 };
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-
-// Every thread of every CTA of the cluster: release this CTA's shared-memory
-// writes (local and remote), then wait for all CTAs (a superset of
-// __syncthreads).
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ uint32_t cluster_addr(const void *local_ptr, uint32_t rank) {
-  const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(local_ptr));
-  uint32_t ra;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
-  return ra;
-}
 // Stores v at local_ptr of CTA `rank`; its 16 bytes count on that CTA's barrier `bar`.
 __device__ __forceinline__ void st_async_f4(const float4 *local_ptr, const uint64_t *bar, uint32_t rank, float4 v) {
   asm volatile(
