@@ -293,7 +293,7 @@ dreams_status_t dreams_vocab_sample(const void *logits, dreams_dtype_t dtype, in
  * decoding"). sample_out ([B, T_max], may be NULL) receives the draws of the
  * rows computed. Three kernel launches, chained by programmatic dependent
  * launch: the two stages of the draws over the node rows, then the walk and
- * the compaction (one CTA per sequence). The workspace holds no state between
+ * the compaction (one CTA per sequence, more for large caches). The workspace holds no state between
  * calls.
  */
 size_t dreams_verify_step_sampled_workspace_size(const dreams_tree_t *tree, int64_t V);
@@ -324,7 +324,8 @@ dreams_status_t dreams_verify_step_sampled(const void *logits, dreams_dtype_t dt
  * out_tokens, new_kv_len and the KV compaction are as in dreams_verify_step.
  * target_logits, draft_logits: f32 or bf16, [B, T_max, V] with row_stride
  * (the same for both); only the rows of the nodes the walk visits are read
- * (the draft row only where children are tried). u_accept, u_resample:
+ * (the draft row only where children are tried; both rows of a visited node's
+ * first child may be prefetched). u_accept, u_resample:
  * device f32 [B, T_max] (the caller's random numbers). Logits must be finite
  * (with non-finite values the tokens drawn are unspecified but lie in
  * [0, V)). V <= 393216 (beyond 196608 the kernel needs clusters of 16 CTAs),

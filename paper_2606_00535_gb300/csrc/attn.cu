@@ -272,7 +272,11 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_c
   __shared__ int s_pair;
 
   grid_wait();
-  launch_successor();
+  // The merge is let in early. Any other successor waits for the exits: the
+  // CTAs end at very different times, and one that streams with a full chip's
+  // worth of CTAs would fill the SMs that end first and leave the others idle
+  // (batched attention and the verification behind it 131.0 against 110.3 us).
+  if (p.nsplit > 1) launch_successor();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int per_pair = p.Hkv * p.nrb;
   const int pair_pos = blockIdx.x / per_pair;
@@ -1007,7 +1011,6 @@ __global__ void __launch_bounds__(256) tree_attn_merge_kernel(const AttnParams p
   const bool live = T >= 1 && T <= p.T_max && L >= 0 && total <= p.capacity && total >= 1 && t0 < T &&
                     r < ::min(p.TB, T - t0) * p.G && nsplit_blk > 1;
   grid_wait();
-  launch_successor();
   if (!live) return;
 
   const int64_t sbase = item * p.nsplit * ROWS + r;

@@ -38,17 +38,21 @@ inline dreams_status_t check_launch() {
 // Every kernel of the library is launched as a programmatic dependent of the
 // launch before it on the stream: its CTAs may become resident while that grid
 // drains, and each begins with grid_wait(), which returns once that grid has
-// completed and its writes are visible. Each then lets its own successor start
-// (launch_successor, after the wait, so that at most one grid ahead of a
-// running CTA is unfinished). Between back-to-back calls this takes the launch
-// gap out. The sampling statistics let it start at the end of their work:
-// successors that took their slots early, or came only with the CTAs' exits,
-// cost 240 rows of 32003 f32 18 against 15 us; the importance sums leave it to
-// the exits (103.3 against 105.3 us), while the attention's merge launched
-// early takes 1.2 us off 18.7. A kernel that reads global memory before its
-// wait may read only what its own predecessor's inputs were (the walk's tree
-// arrays), and reads it through L2 (__ldcg): L1 may hold older lines until the
-// wait.
+// completed and its writes are visible. A kernel whose successor is the next
+// stage of the same call lets it start early (launch_successor, after the wait,
+// so that at most one grid ahead of a running CTA is unfinished): the merge of
+// the attention's partials launched so takes 1.2 us off 18.7. The last kernel
+// of a call leaves its successor to its CTAs' exits: what comes next may stream
+// with a chip's worth of CTAs, which would fill the SMs that are free first and
+// leave the others idle (batched attention, then the verification: 131.0
+// against 110.3 us; a 3392-slot attention and a batched verification 74.8
+// against 57.0).
+// The sampling statistics let the selection start at the end of their work
+// (earlier, or only with the exits, 240 rows of 32003 f32 took 18 against 15
+// us); the importance sums leave it to the exits (103.3 against 105.3 us).
+// A kernel that reads global memory before its wait may read only what its own
+// predecessor's inputs were (the walk's tree arrays), and reads it through L2
+// (__ldcg): L1 may hold older lines until the wait.
 template <typename... Params, typename... Args>
 dreams_status_t launch_clusters(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                                 int cluster, Args... args) {

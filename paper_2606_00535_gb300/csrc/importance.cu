@@ -206,7 +206,6 @@ __global__ void __launch_bounds__(1024) importance_reduce_kernel(const ImpParams
 __global__ void __launch_bounds__(SEL_THREADS) importance_select_kernel(const ImpParams p, int32_t r,
                                                                         const float *importance, int32_t *keep) {
   grid_wait();
-  launch_successor();
   extern __shared__ uint32_t s_key[];
   __shared__ int s_hist[256];
   __shared__ uint32_t s_prefix;

@@ -239,7 +239,6 @@ struct ArgmaxParams {
 template <typename T>
 __global__ void __launch_bounds__(ARGMAX_THREADS) vocab_argmax_kernel(const ArgmaxParams p) {
   grid_wait();
-  launch_successor();
   const int64_t row = blockIdx.x / p.nchunk;
   const int c = blockIdx.x % p.nchunk;
   const T *base = static_cast<const T *>(p.logits) + row * p.row_stride;
@@ -657,7 +656,6 @@ __global__ void __launch_bounds__(256) vocab_sample_select_kernel(const SamplePa
   const int64_t r = int64_t(blockIdx.x) * 8 + (threadIdx.x >> 5);
   const float u = r < rows ? __ldcg(p.u + r) : 0.f;
   grid_wait();
-  launch_successor();
   if (r >= rows) return;
   const int idx = sample_select_warp<T>(p, static_cast<const T *>(p.logits) + r * p.row_stride, p.seg + r * p.nseg, u);
   if ((threadIdx.x & 31) == 0) out[r] = idx;
@@ -909,7 +907,6 @@ __global__ void __launch_bounds__(32) accept_path_kernel(const int32_t *pred, co
                                                          int32_t *accept_len, int32_t *path, int32_t *out_tokens,
                                                          int32_t *new_kv_len, int32_t *status) {
   grid_wait();
-  launch_successor();
   __shared__ int32_t s_path[65];
   const int b = blockIdx.x;
   const int T = __ldg(tr.tree_len + b), L = __ldg(tr.kv_len + b);
@@ -929,7 +926,6 @@ __global__ void __launch_bounds__(TAIL_THREADS) kv_compact_kernel(const KVParams
                                                                   const int32_t *accept_len, const int32_t *path,
                                                                   int max_path, int32_t *status) {
   grid_wait();
-  launch_successor();
   __shared__ int32_t s_path[65];
   __shared__ int64_t s_src[65], s_dst[65];
   __shared__ int s_ok;
@@ -1070,7 +1066,6 @@ __global__ void __launch_bounds__(TAIL_THREADS) verify_tail_kernel(const StepPar
     if (lane < 2) s_pg[lane] = e;
   }
   grid_wait();
-  launch_successor();
   if (threadIdx.x < 32) {
     WalkOut w{-1, 0};
     if (T < 1 || T > Tm) w.bad = DREAMS_DATA_BAD_TREE_LEN;
@@ -1138,15 +1133,16 @@ __global__ void __launch_bounds__(TAIL_THREADS) verify_tail_kernel(const StepPar
 // vocabulary slice [rank * S, (rank + 1) * S) of the rows of the node being
 // visited, as exponentials in shared memory (each thread's relative to its own
 // maximum m, with the factor a = 2^((m - M) k2) to the row's maximum M kept in
-// a register). Only the rows of visited nodes are read. A sum over the
-// vocabulary: warps reduce their threads' values, warp 0 the warps' and sends
+// a register). Only the rows of visited nodes are read (those of a node's first
+// child, tried first, come towards L2 before it is known to be visited). A sum
+// over the vocabulary: warps reduce their threads' values, warp 0 the warps' and sends
 // the CTA's value into every CTA's shared memory (distributed shared memory;
 // asynchronous stores that complete on the receiving CTA's barrier), then each
 // warp combines the cs values in rank order: all CTAs hold bit-identical
 // results, take the same decisions and make the same exchanges. The walk is a
 // chain of such exchanges, so their latency is its time: one store's flight
-// instead of a cluster barrier's arrival and release. The rows' maxima and exponential sums take one such
-// exchange of (maximum, sum) pairs.
+// instead of a cluster barrier's arrival and release. The rows' maxima and
+// exponential sums take one such exchange of (maximum, sum) pairs.
 constexpr int SPEC_THREADS = 512;                    // 16 warps
 constexpr int SPEC_CHUNK = 8 * SPEC_THREADS;         // values per chunk: 8 per thread
 constexpr int SPEC_MAX_J = 6;                        // chunks per CTA slice (192 KB of f32 pairs)
@@ -1499,13 +1495,13 @@ __device__ int spec_slice_draw(SpecShared &sh, const float *et, const float *ed,
 // One cluster of p.cs CTAs per sequence (grid.x = B * cs): the walk with its
 // decisions, the bonus draw, the outputs and the KV compaction. A chain of
 // dependent steps, so its latency is what counts: 16 trees of 32-64 nodes at
-// 128256 bf16 entries took 47.8 us a pass, 32.7 with the root's rows loaded
+// 128256 bf16 entries took 47.8 us a pass, 31.9 with the root's rows loaded
 // under the tree check, exponentials from registers, conflict-free slices, warp
-// maxima by one instruction, and the outputs written by the CTA that draws.
+// maxima by one instruction, the outputs written by the CTA that draws, and the
+// first child's rows prefetched.
 template <typename T>
 __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParams p) {
   grid_wait();
-  launch_successor();
   extern __shared__ __align__(16) float spec_dyn[];
   __shared__ SpecShared sh;
   const int cs = p.cs, J = p.J;
