@@ -244,8 +244,8 @@ dreams_status_t dreams_kv_compact(const dreams_kv_cache_t *kv, int32_t B, const 
  * kv->n_layers layers, with the semantics documented above. argmax_out
  * ([B, T_max], may be NULL) receives the predictions of the rows computed;
  * other rows are untouched. The call makes two kernel launches on the
- * stream: the argmax, then the walk and compaction (one CTA per sequence),
- * chained by programmatic dependent launch.
+ * stream: the argmax, then the walk and compaction (one CTA per sequence, more
+ * for large caches), chained by programmatic dependent launch.
  */
 size_t dreams_verify_step_workspace_size(const dreams_tree_t *tree, int64_t V);
 dreams_status_t dreams_verify_step(const void *logits, dreams_dtype_t dtype, int64_t V,
@@ -293,8 +293,8 @@ dreams_status_t dreams_vocab_sample(const void *logits, dreams_dtype_t dtype, in
  * decoding"). sample_out ([B, T_max], may be NULL) receives the draws of the
  * rows computed. Three kernel launches, chained by programmatic dependent
  * launch: the two stages of the draws over the node rows, then the walk and
- * the compaction (one CTA per sequence, more for large caches). The workspace holds no state between
- * calls.
+ * the compaction (one CTA per sequence, more for large caches). The workspace
+ * holds no state between calls.
  */
 size_t dreams_verify_step_sampled_workspace_size(const dreams_tree_t *tree, int64_t V);
 dreams_status_t dreams_verify_step_sampled(const void *logits, dreams_dtype_t dtype, int64_t V,

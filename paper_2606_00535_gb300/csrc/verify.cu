@@ -25,8 +25,8 @@
 // batch in increasing x) never overwrites a slot it still has to read.
 //
 // The fused step is two launches: the argmax over the rows of real tree nodes,
-// then, one CTA per sequence and chained by programmatic dependent launch, the
-// walk and the compaction. Kept apart, the argmax kernel needs few registers,
+// then, one CTA per sequence (more for large caches) and chained by programmatic
+// dependent launch, the walk and the compaction. Kept apart, the argmax kernel needs few registers,
 // so every CTA of a large batch is resident at once.
 #include <limits.h>
 
