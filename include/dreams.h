@@ -31,6 +31,8 @@
  *    zero-fill such a workspace once when it is allocated, and every call
  *    leaves it zero-filled again, whatever its shape arguments. Calls that
  *    overlap in time must not share a workspace.
+ *  - new_kv_len may be the tree's kv_len array itself: a decode loop may
+ *    advance its lengths in place.
  *  - Every call is asynchronous on the given stream (NULL = the legacy
  *    default stream) and runs on the current CUDA device.
  *  - Host-side checks (null pointers, sizes, alignment, supported shapes)

@@ -970,6 +970,8 @@ struct StepParams {
   KVParams kv;
   int32_t max_path;
   int32_t ntail;  // CTAs per sequence of the walk and compaction launch
+  int32_t *ticket;      // with ntail > 1: sequence b's CTAs that have read their inputs, at ticket[b * ticket_step]
+  int64_t ticket_step;  // (zero before that launch)
   int32_t *pred;  // [B, T_max] predictions (caller's argmax_out or workspace)
   bool pred_in_ws;
   int32_t *accept_len, *path, *out_tokens, *new_kv_len;
@@ -1028,37 +1030,51 @@ __global__ void __launch_bounds__(256) verify_sample_select_kernel(const StepPar
   const float u = b < p.tr.B ? __ldcg(p.sp.u + r) : 0.f;
   grid_wait();
   launch_successor();
-  if (b >= p.tr.B || tl < 1 || tl > p.tr.T_max || i >= tl) return;
-  const int idx = sample_select_warp<T>(p.sp, static_cast<const T *>(p.sp.logits) + r * p.sp.row_stride,
-                                        p.sp.seg + r * p.sp.nseg, u);
-  if ((threadIdx.x & 31) == 0) p.pred[r] = idx;
+  if (b >= p.tr.B) return;
+  if (tl >= 1 && tl <= p.tr.T_max && i < tl) {
+    const int idx = sample_select_warp<T>(p.sp, static_cast<const T *>(p.sp.logits) + r * p.sp.row_stride,
+                                          p.sp.seg + r * p.sp.nseg, u);
+    if ((threadIdx.x & 31) == 0) p.pred[r] = idx;
+  }
+  // the statistics of the sequence's first row, read by this warp alone, make
+  // room for the tail's counter
+  if (p.ntail > 1 && i == 0) {
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) p.ticket[b * p.ticket_step] = 0;
+  }
 }
 
 // Launch 2 of the verification tail, p.ntail CTAs per sequence, chained to
 // launch 1 by programmatic dependent launch (it may start early and waits
 // until launch 1 has completed): the acceptance walk, its outputs, and the KV
 // compaction. Every CTA of a sequence does the same walk (a warp's work on 64
-// predictions); the first writes the outputs, and the compaction's 16-byte
-// columns, of which a whole model's cache has thousands, are spread over all
-// of them: the moves are latency-bound, so one CTA going through the columns
-// of 32 layers x 32 heads took 50 us where the spread takes the time of one
-// batch of moves (see tail_ctas for the sizes).
+// predictions), and the compaction's 16-byte columns, of which a whole model's
+// cache has thousands, are spread over all of them: the moves are
+// latency-bound, so one CTA going through the columns of 32 layers x 32 heads
+// took 50 us where the spread takes the time of one batch of moves (see
+// tail_ctas for the sizes). The CTA that is the last of its sequence to have
+// read lengths, tree and predictions writes the outputs and clears predictions
+// kept in the workspace: a caller may advance its lengths in place
+// (new_kv_len == kv_len), and a CTA that starts late must not read the new one.
 __global__ void __launch_bounds__(TAIL_THREADS) verify_tail_kernel(const StepParams p) {
   __shared__ int32_t s_path[65], s_out[65], s_pg[2];
   __shared__ int64_t s_src[65], s_dst[65];
   __shared__ int s_n;
   const int b = blockIdx.x / p.ntail, part = blockIdx.x % p.ntail, Tm = p.tr.T_max;
   const int64_t rb = int64_t(b) * Tm;
-  const int T = __ldcg(p.tr.tree_len + b);
-  const int L = __ldcg(p.tr.kv_len + b);
+  // Warp 0 does all but the moves; only it reads the sequence's inputs.
   // Everything that needs no prediction is done while the argmax grid runs:
   // the tree's shape (with its tokens, which the walk then emits from
   // registers) and, for a paged cache, the page-table entries of the tree's
-  // slots L .. L + T - 1 (two pages at most), which the compaction needs.
-  const bool lens_ok = T >= 1 && T <= Tm && L >= 0 && L <= p.kv.capacity - T;
+  // slots.
+  int T = 0, L = 0;
+  bool lens_ok = false;
   TreeShape ts{};
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
+    T = __ldcg(p.tr.tree_len + b);
+    L = __ldcg(p.tr.kv_len + b);
+    lens_ok = T >= 1 && T <= Tm && L >= 0 && L <= p.kv.capacity - T;
     int e = -1;
     if (lane < 2 && lens_ok && p.kv.page_table != nullptr && (L >> 6) + lane < p.kv.pages_per_seq)
       e = __ldcg(p.kv.page_table + int64_t(b) * p.kv.pages_per_seq + (L >> 6) + lane);
@@ -1066,44 +1082,46 @@ __global__ void __launch_bounds__(TAIL_THREADS) verify_tail_kernel(const StepPar
     if (lane < 2) s_pg[lane] = e;
   }
   grid_wait();
+  WalkOut w{-1, 0};
+  int ticket = 0;
+  auto write_outputs = [&]() {
+    write_walk(b, w.n, L, p.tr.tokens + rb, p.pred + rb, s_path, p.max_path, p.accept_len, p.path, p.out_tokens,
+               p.new_kv_len, s_out);
+    if (p.pred_in_ws && T >= 1 && T <= Tm)  // leave the workspace zero-filled
+      for (int x = threadIdx.x; x < T; x += 32) p.pred[rb + x] = 0;
+  };
   if (threadIdx.x < 32) {
-    WalkOut w{-1, 0};
     if (T < 1 || T > Tm) w.bad = DREAMS_DATA_BAD_TREE_LEN;
-    else if (L < 0 || L > p.kv.capacity - T) w.bad = DREAMS_DATA_BAD_KV_LEN;
+    else if (!lens_ok) w.bad = DREAMS_DATA_BAD_KV_LEN;
     else if (ts.bad) w.bad = ts.bad;
     else w = tree_walk_finish(ts, p.pred + rb, T, p.max_path, s_path, s_out);
     if (w.bad) {
       w.n = -1;
       if (part == 0 && threadIdx.x == 0) flag(p.status, w.bad);
     }
-    if (part == 0)
-      write_walk(b, w.n, L, p.tr.tokens + rb, p.pred + rb, s_path, p.max_path, p.accept_len, p.path, p.out_tokens,
-                 p.new_kv_len, s_out);
-    if (p.pred_in_ws && T >= 1 && T <= Tm) {
-      // leave the workspace zero-filled: the CTA that read the predictions
-      // last (a count on the sequence's first row counter, zero again since
-      // the argmax grid completed) clears them
-      int last = 1;
-      if (p.ntail > 1) {
-        __threadfence();
-        __syncwarp();
-        if (threadIdx.x == 0) {
-          last = atomicAdd(p.am.cnt + rb, 1) == p.ntail - 1;
-          if (last) p.am.cnt[rb] = 0;
-        }
-        last = __shfl_sync(0xffffffffu, last, 0);
-      }
-      __syncwarp();
-      for (int x = threadIdx.x; last && x < T; x += 32) p.pred[rb + x] = 0;
-    }
     bool ok = w.n > 0;
     if (ok) ok = move_offsets(p.kv, b, L, w.n, s_path, s_src, s_dst, part == 0 ? p.status : nullptr, s_pg);
     if (threadIdx.x == 0) s_n = ok ? w.n : 0;
+    if (p.ntail == 1) {
+      __syncwarp();
+      write_outputs();
+    }
   }
   __syncthreads();
+  // (the ticket's round trip runs under the moves)
+  if (p.ntail > 1 && threadIdx.x < 32) {
+    __threadfence();
+    __syncwarp();
+    if (threadIdx.x == 0) ticket = atomicAdd(p.ticket + b * p.ticket_step, 1);
+  }
   const int n = s_n;
   if (n > 0)
     compact_units(p.kv, n, s_src, s_dst, part * int64_t(blockDim.x) + threadIdx.x, int64_t(p.ntail) * blockDim.x);
+  if (p.ntail > 1 && threadIdx.x < 32 && __shfl_sync(0xffffffffu, ticket, 0) == p.ntail - 1) {
+    __threadfence();
+    write_outputs();
+    if (threadIdx.x == 0) p.ticket[b * p.ticket_step] = 0;
+  }
 }
 
 // ------------------------------------------------------------------ speculative sampling
@@ -1951,6 +1969,8 @@ extern "C" dreams_status_t dreams_verify_step(const void *logits, dreams_dtype_t
   p.pred = argmax_out != nullptr ? argmax_out : ws_pred;
   p.pred_in_ws = argmax_out == nullptr;
   p.ntail = tail_ctas(p.kv, tree->B);
+  p.ticket = p.am.cnt;  // the row counters, zero again once the argmax grid has completed
+  p.ticket_step = tree->T_max;
   p.max_path = max_path;
   p.accept_len = accept_len;
   p.path = path;
@@ -2028,6 +2048,8 @@ extern "C" dreams_status_t dreams_verify_step_sampled(
   p.pred = sample_out != nullptr ? sample_out : ws_pred;
   p.pred_in_ws = false;
   p.ntail = tail_ctas(p.kv, tree->B);
+  p.ticket = reinterpret_cast<int32_t *>(p.sp.seg);  // each sequence's first statistics, cleared by the selection
+  p.ticket_step = int64_t(tree->T_max) * p.sp.nseg * 2;
   p.max_path = max_path;
   p.accept_len = accept_len;
   p.path = path;
