@@ -340,7 +340,9 @@ dreams_status_t dreams_verify_step_sampled(const void *logits, dreams_dtype_t dt
  * sequence, each holding a slice of the visited node's rows in shared memory;
  * a rejection costs one sum over the slices, combined across the cluster in
  * distributed shared memory. The cluster then draws the bonus, writes the
- * outputs and moves the accepted K/V.
+ * outputs and moves the accepted K/V. A wait of the cluster's CTAs for one
+ * another that times out flags DREAMS_DATA_TIMEOUT; the outputs and the cache
+ * of that sequence are then left untouched.
  */
 dreams_status_t dreams_verify_step_speculative(const void *target_logits, const void *draft_logits,
                                                dreams_dtype_t dtype, int64_t V, int64_t row_stride,
@@ -429,9 +431,9 @@ dreams_status_t dreams_vocab_argmax_noalloc(const void *logits, dreams_dtype_t d
                                             int64_t row_stride, int32_t *out_idx, dreams_stream_t stream);
 
 /*
- * Test hook for the bounded pipeline waits of the tcgen05 kernels; not for
- * production use. The paper has no counterpart: every wait of these kernels
- * on its own copy or MMA pipeline gives up after a limit instead of hanging
+ * Test hook for the bounded waits of the tcgen05 kernels and the speculative
+ * walk; not for production use. The paper has no counterpart: every wait of these kernels
+ * on its own copies, MMAs or exchanges gives up after a limit instead of hanging
  * the GPU, and this hook lets a test make such a wait run out without any
  * fault. While stall_at >= 0, every later launch of the kernels selected by
  * `kernels` (DREAMS_TEST_ATTENTION: dreams_tree_verify_attn and
@@ -443,12 +445,16 @@ dreams_status_t dreams_vocab_argmax_noalloc(const void *logits, dreams_dtype_t d
  * DREAMS_DATA_TIMEOUT, wait for the copies and MMAs they did issue, free
  * their tensor memory and exit; output rows they did not finish are left
  * untouched (attention), or unreliable (LM head; rows no tile reached are
- * untouched). stall_at < 0 restores normal operation (the other arguments
+ * untouched). DREAMS_TEST_SPECULATIVE (dreams_verify_step_speculative)
+ * withholds nothing, but lets the first CTA of each cluster wait for one value
+ * too many in exchange stall_at of the walk (0: the root's maxima and sums; a
+ * rejection and a further node take one more each). stall_at < 0 restores normal operation (the other arguments
  * are then ignored). The setting is process-wide and read at launch, so a
  * CUDA graph keeps the setting it was captured with.
  */
 #define DREAMS_TEST_ATTENTION 1
 #define DREAMS_TEST_LM_HEAD 2
+#define DREAMS_TEST_SPECULATIVE 8
 dreams_status_t dreams_test_set_stall(int32_t kernels, int32_t stall_at, int64_t wait_limit_ns);
 
 const char *dreams_status_string(dreams_status_t status);

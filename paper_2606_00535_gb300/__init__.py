@@ -35,7 +35,7 @@ NOALLOC_ARGMAX_MAX_ROWS = 16384
 F32, BF16 = 0, 1
 DATA_BAD_PARENT, DATA_BAD_TREE_LEN, DATA_BAD_KV_LEN, DATA_BAD_PAGE, DATA_BAD_PATH = 1, 2, 4, 8, 16
 DATA_TIMEOUT = 0x20  # a kernel gave up waiting on its own pipeline
-TEST_ATTENTION, TEST_LM_HEAD = 1, 2  # kernel families of test_set_stall
+TEST_ATTENTION, TEST_LM_HEAD, TEST_SPECULATIVE = 1, 2, 8  # kernel families of test_set_stall
 
 
 class DreamsError(RuntimeError):

@@ -98,8 +98,11 @@ __device__ __forceinline__ uint32_t cluster_rank() {
 // Every thread of every CTA of the cluster: release this CTA's shared-memory
 // writes (local and remote), then wait for all CTAs (a superset of
 // __syncthreads).
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  cluster_arrive();
+  cluster_wait();
 }
 
 __device__ __forceinline__ uint32_t cluster_addr(const void *local_ptr, uint32_t rank) {

@@ -1159,8 +1159,13 @@ __global__ void __launch_bounds__(TAIL_THREADS) verify_tail_kernel(const StepPar
 // warp combines the cs values in rank order: all CTAs hold bit-identical
 // results, take the same decisions and make the same exchanges. The walk is a
 // chain of such exchanges, so their latency is its time: one store's flight
-// instead of a cluster barrier's arrival and release. The rows' maxima and
-// exponential sums take one such exchange of (maximum, sum) pairs.
+// instead of a cluster barrier's arrival and release (four trees whose
+// root's drafts are rejected, at 128256 bf16 entries, 14.4 us against 15.8, one
+// tree of accepted ones 17.8 against 18.4). The rows' maxima and exponential sums take one such exchange of
+// (maximum, sum) pairs. An exchange that does not arrive within the limit ends
+// the walk of the whole cluster with nothing written: the CTA's warps agree on
+// it by a vote, and the CTAs by a cluster barrier before the outputs, whose
+// arrival goes ahead of the bonus draw.
 constexpr int SPEC_THREADS = 512;                    // 16 warps
 constexpr int SPEC_CHUNK = 8 * SPEC_THREADS;         // values per chunk: 8 per thread
 constexpr int SPEC_MAX_J = 6;                        // chunks per CTA slice (192 KB of f32 pairs)
@@ -1178,8 +1183,14 @@ struct SpecParams {
   const float *u_acc, *u_res;  // [B, T_max] each
   int32_t *accept_len, *path, *out_tokens, *new_kv_len;
   int32_t *status;
+  uint64_t wait_ns;  // limit of an exchange's wait (2 s unless a test shortens it)
+  int32_t stall_at;  // test hook: the first CTA expects one partial too many of this exchange (-1: off)
 };
 
+// Sets *local_ptr of CTA `rank` to 1.
+__device__ __forceinline__ void st_cluster_one(const int32_t *local_ptr, uint32_t rank) {
+  asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(cluster_addr(local_ptr, rank)), "r"(1) : "memory");
+}
 // Stores v at local_ptr of CTA `rank`; its 16 bytes count on that CTA's barrier `bar`.
 __device__ __forceinline__ void st_async_f4(const float4 *local_ptr, const uint64_t *bar, uint32_t rank, float4 v) {
   asm volatile(
@@ -1188,10 +1199,13 @@ __device__ __forceinline__ void st_async_f4(const float4 *local_ptr, const uint6
       "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(cluster_addr(bar, rank))
       : "memory");
 }
+
 struct SpecShared {
   float4 slot[2][SPEC_MAX_CS];       // [parity][rank]: every CTA's partial of the current exchange
   uint64_t bar[2];                   // [parity]: the exchange's cs partials have arrived
-  int32_t zero, late;                // (never set; an exchange did not arrive in time)
+  int32_t zero;                      // (never set)
+  int32_t votes;                     // warps whose wait for the current exchange has run out
+  int32_t dead;                      // a CTA of the cluster gave the walk up
   float chunk[SPEC_MAX_J][16];       // the bonus draw: per-warp sums of each chunk
   float red[16];                     // the bonus draw: per-warp sums of the slice
   float4 red4[16];                   // per-warp partials of a sum or of (maximum, sum) pairs
@@ -1253,49 +1267,93 @@ __device__ __forceinline__ float4 ms4_lanes(float4 v, float k2) {
 }
 
 // One exchange of the cluster, number x (0, 1, ...): warp 0's lane r sends this
-// CTA's partial to CTA r, and every thread waits for the cs partials sent to
-// its own CTA. Exchanges alternate between two sets of slots and barriers: a
-// CTA sends number x + 2 only once it holds every partial of x + 1, and those
-// were sent after their senders' threads had read the slots of x.
-__device__ __forceinline__ void spec_send(SpecShared &sh, float4 cta, int x, int cs, uint32_t rank) {
+// CTA's partial to CTA r, and every warp waits for the cs partials sent to its
+// own CTA. Exchanges alternate between two sets of slots and barriers: a CTA
+// sends number x + 2 only once it holds every partial of x + 1, and those were
+// sent after their senders' threads had read the slots of x. (The bonus's is
+// the one exchange that the test hook leaves whole.)
+__device__ __forceinline__ void spec_send(SpecShared &sh, const SpecParams &p, float4 cta, int x, uint32_t rank,
+                                          bool bonus = false) {
   const int lane = threadIdx.x & 31;
-  if (lane == 0) tc::mbar_arrive_expect_tx(smem_u32(&sh.bar[x & 1]), uint32_t(cs) * 16u);
-  if (lane < cs) st_async_f4(&sh.slot[x & 1][rank], &sh.bar[x & 1], uint32_t(lane), cta);
+  const uint32_t extra = !bonus && x == p.stall_at && rank == 0 ? 16u : 0u;
+  if (lane == 0) tc::mbar_arrive_expect_tx(smem_u32(&sh.bar[x & 1]), uint32_t(p.cs) * 16u + extra);
+  if (lane < p.cs) st_async_f4(&sh.slot[x & 1][rank], &sh.bar[x & 1], uint32_t(lane), cta);
 }
-__device__ __forceinline__ void spec_arrived(SpecShared &sh, int x) {
-  const uint32_t bar = smem_u32(&sh.bar[x & 1]);
-  if (!tc::mbar_wait_cluster(bar, (x >> 1) & 1, &sh.zero)) sh.late = 1;  // (after 2 s: flagged at the end)
+
+// A warp's wait ran out. Whether the walk is given up must be one answer for the
+// CTA, whose warps meet in barriers, so the warp votes and goes on looking:
+// false once all have voted; true if the exchange arrives after all, after
+// taking the vote back, which is possible only while some warp has not voted. A
+// warp that never voted saw the exchange arrive, so the others will too. (No
+// warp can be an exchange ahead: the next one has a barrier of the CTA before
+// its wait.)
+__device__ __noinline__ bool spec_vote(int32_t *votes, uint32_t bar, uint32_t parity) {
+  const bool lead = (threadIdx.x & 31) == 0;
+  if (lead) atomicAdd(votes, 1);
+  for (;;) {
+    int v = lead ? *static_cast<volatile int32_t *>(votes) : 0;
+    if (__shfl_sync(0xffffffffu, v, 0) == SPEC_THREADS / 32) return false;
+    if (!__all_sync(0xffffffffu, tc::mbar_try_wait_cluster(bar, parity))) continue;
+    bool back = false;
+    while (lead && !back && v < SPEC_THREADS / 32) {
+      const int was = atomicCAS(votes, v, v - 1);
+      back = was == v;
+      v = was;
+    }
+    if (__any_sync(0xffffffffu, back)) return true;
+  }
+}
+
+// Waits for exchange x: true, or on every thread of the CTA false when it did
+// not arrive within the limit.
+__device__ __forceinline__ bool spec_arrived(SpecShared &sh, const SpecParams &p, int x) {
+  const uint32_t bar = smem_u32(&sh.bar[x & 1]), parity = (x >> 1) & 1;
+  uint64_t t0 = 0;
+  for (uint32_t it = 0;; ++it) {
+    if (__all_sync(0xffffffffu, tc::mbar_try_wait_cluster(bar, parity))) return true;
+    if ((it & 255u) == 255u) {
+      const uint64_t now = tc::global_ns();
+      if (it == 255u) t0 = now;
+      if (__any_sync(0xffffffffu, now - t0 > p.wait_ns)) break;
+    }
+  }
+  return spec_vote(&sh.votes, bar, parity);
 }
 
 // A sum over the cluster: warps, then warp 0 over the warps, then the CTAs'
 // values, combined in rank order on every warp (the same bits everywhere).
-__device__ __forceinline__ float spec_cluster_sum(SpecShared &sh, float v, int x, int cs, uint32_t rank) {
+// False when the exchange did not arrive.
+__device__ __forceinline__ bool spec_cluster_sum(SpecShared &sh, const SpecParams &p, float v, int x, uint32_t rank,
+                                                 float &sum) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float wv = warp_sum_bcast(v);
   if (lane == 0) sh.red[warp] = wv;
   __syncthreads();
   if (warp == 0) {
     const float cta = warp_sum_bcast(lane < 16 ? sh.red[lane] : 0.f);
-    spec_send(sh, make_float4(cta, 0.f, 0.f, 0.f), x, cs, rank);
+    spec_send(sh, p, make_float4(cta, 0.f, 0.f, 0.f), x, rank);
   }
-  spec_arrived(sh, x);
-  return warp_sum_bcast(lane < cs ? sh.slot[x & 1][lane].x : 0.f);
+  if (!spec_arrived(sh, p, x)) return false;
+  sum = warp_sum_bcast(lane < p.cs ? sh.slot[x & 1][lane].x : 0.f);
+  return true;
 }
 
 // The rows' maxima and exponential sums over the cluster from each thread's
 // (m_t, s_t, m_d, s_d), s = sum 2^((x - m) k2): (Mt, Zt, Md, Zd). The same
 // three levels as a sum: warps, warp 0 over the warps, the CTAs.
-__device__ float4 spec_cluster_ms(SpecShared &sh, float4 v, int x, int cs, uint32_t rank, float k2) {
+__device__ __forceinline__ bool spec_cluster_ms(SpecShared &sh, const SpecParams &p, float4 v, int x, uint32_t rank,
+                                                float4 &ms) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const float4 w = ms4_lanes(v, k2);
+  const float4 w = ms4_lanes(v, p.k2);
   if (lane == 0) sh.red4[warp] = w;
   __syncthreads();
   if (warp == 0) {
-    const float4 cta = ms4_lanes(lane < 16 ? sh.red4[lane] : make_float4(-INFINITY, 0.f, -INFINITY, 0.f), k2);
-    spec_send(sh, cta, x, cs, rank);
+    const float4 cta = ms4_lanes(lane < 16 ? sh.red4[lane] : make_float4(-INFINITY, 0.f, -INFINITY, 0.f), p.k2);
+    spec_send(sh, p, cta, x, rank);
   }
-  spec_arrived(sh, x);
-  return ms4_lanes(lane < cs ? sh.slot[x & 1][lane] : make_float4(-INFINITY, 0.f, -INFINITY, 0.f), k2);
+  if (!spec_arrived(sh, p, x)) return false;
+  ms = ms4_lanes(lane < p.cs ? sh.slot[x & 1][lane] : make_float4(-INFINITY, 0.f, -INFINITY, 0.f), p.k2);
+  return true;
 }
 
 // Warp 0: the parent and token rows of a sequence into sh (entries past
@@ -1519,9 +1577,19 @@ __device__ int spec_slice_draw(SpecShared &sh, const float *et, const float *ed,
 // first child's rows prefetched.
 template <typename T>
 __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParams p) {
-  grid_wait();
   extern __shared__ __align__(16) float spec_dyn[];
   __shared__ SpecShared sh;
+  // this CTA's barriers are ready for the others' partials (they wait for this
+  // arrival before their first exchange)
+  if (threadIdx.x == 0) {
+    tc::mbar_init(smem_u32(&sh.bar[0]), 1);
+    tc::mbar_init(smem_u32(&sh.bar[1]), 1);
+    tc::fence_barrier_init();
+    sh.zero = sh.votes = sh.dead = 0;
+  }
+  __syncthreads();
+  cluster_arrive();
+  grid_wait();
   const int cs = p.cs, J = p.J;
   const uint32_t rank = cluster_rank();
   const int b = int(blockIdx.x / cs);
@@ -1551,12 +1619,6 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
   uint4 wt[SPEC_MAX_J][sizeof(T) / 2], wd[PAIR ? SPEC_MAX_J : 1][PAIR ? sizeof(T) / 2 : 1];
   spec_issue<T>(p, static_cast<const T *>(p.tgt) + rb * p.row_stride, v0, wt);
   if constexpr (PAIR) spec_issue<T>(p, static_cast<const T *>(p.drf) + rb * p.row_stride, v0, wd);
-  if (tid == 0) {
-    tc::mbar_init(smem_u32(&sh.bar[0]), 1);
-    tc::mbar_init(smem_u32(&sh.bar[1]), 1);
-    tc::fence_barrier_init();
-    sh.zero = sh.late = 0;
-  }
   if (warp == 0) {
     int bad = 0;
     if (TL < 1 || TL > Tm) bad = DREAMS_DATA_BAD_TREE_LEN;
@@ -1574,9 +1636,12 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
       if (bad && rank == 0) flag(p.status, bad);
     }
   }
-  cluster_sync();  // every CTA's barriers are ready for the others' partials
+  __syncthreads();
+  cluster_wait();
   const bool bad = sh.cmd != 0;
-  int n = -1, bonus = 0, xc = 0;  // xc: exchanges made
+  int n = -1, bonus = 0, xc = 0;  // xc: exchanges that have arrived
+  bool dead = false;              // one did not
+  bool sent = false, agreed = false;  // arrived at the cluster's last barrier; past it
   int writer = 0;  // the CTA that draws the bonus and writes the outputs
   if (!bad) {
     int cur = 0;
@@ -1628,7 +1693,10 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
         }
       }
       const float2 m = make_float2(mt.x, md.x);
-      const float4 g = spec_cluster_ms(sh, make_float4(m.x, mt.y, m.y, md.y), xc++, cs, rank, k2);
+      float4 g;
+      dead = !spec_cluster_ms(sh, p, make_float4(m.x, mt.y, m.y, md.y), xc, rank, g);
+      if (dead) break;
+      ++xc;
       const float Mt = g.x, Zd = g.w;
       // this thread's factors to the rows' maxima (its exponentials are
       // relative to its own maxima), and their ratio for the passes
@@ -1659,9 +1727,13 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
             acc1 += spec_w(tv.z, dv.z, ct) + spec_w(tv.w, dv.w, ct);
           }
         }
-        const float Pn = spec_cluster_sum(sh, at * (acc0 + acc1), xc++, cs, rank);
+        float Pn;
+        dead = !spec_cluster_sum(sh, p, at * (acc0 + acc1), xc, rank, Pn);
+        if (dead) break;
+        ++xc;
         if (Pn > 0.f) c = c2, Pu = Pn;  // a zero sum (r == q) keeps the residual
       }
+      if (dead) break;
       if (next >= 0) {
         ++n;
         cur = next;
@@ -1684,12 +1756,21 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
         __syncthreads();
         if (warp == 0) {
           const float slice = warp_sum_bcast(lane < 16 ? sh.red[lane] : 0.f);
-          spec_send(sh, make_float4(slice, 0.f, 0.f, 0.f), xc, cs, rank);
+          spec_send(sh, p, make_float4(slice, 0.f, 0.f, 0.f), xc, rank, true);
         }
-        spec_arrived(sh, xc);
+        __syncwarp();
+        cluster_arrive();  // this CTA has had all exchanges but this, which it has sent
+        sent = true;
+        if (!spec_arrived(sh, p, xc)) {
+          // some CTA gave up before, or (all having sent theirs) it only has to land
+          cluster_wait();
+          agreed = true;
+          const uint32_t bar = smem_u32(&sh.bar[xc & 1]);
+          dead = sh.dead || !__syncthreads_and(tc::mbar_wait_cluster(bar, (xc >> 1) & 1, &sh.zero, p.wait_ns));
+          if (dead) break;
+        }
       }
       const float tr = lane < cs ? sh.slot[xc & 1][lane].x : 0.f;
-      ++xc;
       // their running sum across the lanes, then the crossing slice
       float inc = tr;
 #pragma unroll
@@ -1717,9 +1798,24 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
       break;
     }
   }
+  // Nothing is written before every CTA of the cluster has had all exchanges but
+  // the bonus's and has sent that. A CTA that gave up tells the others (those it
+  // left without its partials give up in turn); all then leave outputs and cache
+  // alone, and end only after the limit once more, when nothing sent to them
+  // can still be under way.
+  if (!sent) {
+    if (dead && tid < cs) st_cluster_one(&sh.dead, uint32_t(tid));
+    __syncwarp();
+    cluster_arrive();
+  }
+  if (!agreed) cluster_wait();
+  if (dead || sh.dead) {
+    if (tid == 0) flag(p.status, DREAMS_DATA_TIMEOUT);
+    tc::mbar_wait_cluster(smem_u32(&sh.bar[xc & 1]), (xc >> 1) & 1, &sh.zero, p.wait_ns);
+    return;
+  }
   // outputs: path, drafts then the bonus, lengths; the compaction is shared by
-  // the cluster's CTAs. (No CTA leaves early: its last exchange brought it every
-  // partial that was ever sent to it.)
+  // the cluster's CTAs
   if (warp == 0) {
     if (int(rank) == writer) {
       const int mp = p.max_path;
@@ -1737,7 +1833,6 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
         p.new_kv_len[b] = n >= 0 ? L + n + 1 : L;
       }
     }
-    if (lane == 0 && sh.late) flag(p.status, DREAMS_DATA_TIMEOUT);
     bool ok = n > 0;
     if (ok) ok = move_offsets(p.kv, b, L, n, sh.path, sh.src, sh.dst, rank == 0 ? p.status : nullptr, sh.pg);
     if (lane == 0) sh.cmd = ok ? n : 0;
@@ -2103,6 +2198,7 @@ extern "C" dreams_status_t dreams_verify_step_speculative(
   p.out_tokens = out_tokens;
   p.new_kv_len = new_kv_len;
   p.status = status_word;
+  test_stall(DREAMS_TEST_SPECULATIVE, &p.stall_at, &p.wait_ns);
   const int smem = pl.J * SPEC_CHUNK * 2 * int(sizeof(float));
   void (*kernel)(const SpecParams) =
       dtype == DREAMS_F32 ? spec_walk_kernel<float> : spec_walk_kernel<__nv_bfloat16>;

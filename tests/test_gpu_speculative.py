@@ -405,3 +405,48 @@ def test_speculative_llava_f32_temperature_1(dreams, seed):
                  w.max_path, 1.0, u_acc, u_res)
     assert st == 0
     _compare(r, ref)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("B, V", [(3, 3000), (3, 9001), (3, 20000), (5, 40000), (2, 128256)])
+def test_speculative_many_exchanges(dreams, dtype, B, V):
+    """Clusters of 1, 2, 4, 8 and 16 CTAs through about 65 exchanges each: the
+    root's 31 children and the last one's 32 are rejected one after the other
+    down to the last of each, whose acceptance needs the residual left by all
+    the others. Twenty walks in a row, all equal to the oracle's."""
+    rng = np.random.default_rng(V + (dtype == "bf16"))
+    T, tau = 64, 1.0
+    tgt32 = rng.standard_normal((B, T, V), dtype=np.float32) * 2
+    tgt32[:, 63] *= 2  # the bonus is drawn among a few wide entries
+    drf32 = tgt32 + rng.standard_normal((B, T, V), dtype=np.float32) * np.float32(0.8)
+    par = np.full((B, T), -1, np.int32)
+    par[:, 1:32], par[:, 32:] = 0, 31
+    tok = np.zeros((B, T), np.int32)
+    u_acc = np.full((B, T), 0.9999, np.float32)
+    u_acc[:, [31, 63]] = 0.0
+    for b in range(B):
+        for node, kids in ((0, range(1, 32)), (31, range(32, 64))):
+            order = np.argsort(tgt32[b, node] - drf32[b, node])
+            tok[b, kids] = order[:len(kids)]  # where the draft says most too much
+            tok[b, kids[-1]] = order[-1]      # and least
+    tl, kl = np.full(B, T, np.int32), rng.integers(0, 30, B).astype(np.int32)
+    if dtype == "bf16":
+        tgt_t, drf_t = W.bf16(tgt32), W.bf16(drf32)
+        tgt_np, drf_np = W.bits(tgt_t), W.bits(drf_t)
+    else:
+        tgt_t, drf_t = torch.from_numpy(tgt32), torch.from_numpy(drf32)
+        tgt_np, drf_np = tgt32, drf32
+    for _ in range(60):  # the bonus away from its thresholds
+        u_res = rng.random((B, T), dtype=np.float32)
+        ref = oracle.spec_path(tgt_np, drf_np, par, tok, tl, kl, 6, tau, u_acc, u_res, bf16_bits=dtype == "bf16")
+        if (ref["margin"] > MARGIN).all():
+            break
+    assert (ref["margin"] > MARGIN).all() and (ref["path"][:, :3] == [0, 31, 63]).all()
+    k = torch.zeros((B, 128, 1, 64), dtype=torch.bfloat16, device="cuda")
+    kv = dreams.KVCache(k, k.clone())
+    f = lambda a: torch.from_numpy(a).cuda()  # noqa: E731
+    tree, tgt_t, drf_t, ua, ur, st = (dreams.Tree(f(par), f(tok), f(tl), f(kl)), tgt_t.cuda(), drf_t.cuda(), f(u_acc),
+                                      f(u_res), _status())
+    for r in [dreams.verify_step_speculative(tgt_t, drf_t, tree, kv, 6, tau, ua, ur, status=st) for _ in range(20)]:
+        _compare(r, ref)
+    assert int(st.item()) == 0

@@ -1,12 +1,13 @@
-"""The bounded pipeline waits of the tcgen05 kernels, made to run out on
-purpose without any fault: the test hook dreams_test_set_stall withholds the
+"""The bounded waits of the tcgen05 kernels and of the speculative walk, made to
+run out on purpose without any fault: the test hook dreams_test_set_stall withholds the
 TMA copies of each CTA from a given tile on (the consumers then wait on
 barriers that nothing completes) and shortens every wait to 20 ms. The kernels
 must flag DREAMS_DATA_TIMEOUT, leave the output rows they did not finish
 untouched, wait for the copies and MMAs they did issue and free their tensor
 memory: the next normal call on the same device must then be bit-identical to
 a call made before the stall (a CTA that kept its tensor memory would leave the
-next kernel unable to allocate)."""
+next kernel unable to allocate). In one of the walk's exchanges the first CTA of
+each cluster waits in vain: no CTA of such a cluster may write."""
 import numpy as np
 import pytest
 import torch
@@ -134,3 +135,59 @@ def test_lm_head_wait_runs_out_then_recovers(dreams):
         dreams.test_set_stall(0, -1)
     idx2, mx2, st2 = run()
     assert st2 == 0 and torch.equal(idx2, ref_idx) and torch.equal(mx2, ref_mx)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("V", [777, 20000, 128256])  # clusters of 1, 4 and 16
+def test_speculative_wait_runs_out_then_recovers(dreams, V, dtype):
+    """Chains whose every draft is accepted, behind a first child that is not: a
+    walk of n drafts makes n + 2 exchanges that can be late (each visited node's
+    rows, the rejection; not the bonus's). With exchange x incomplete for one CTA, sequences that
+    reach it keep their outputs and every byte of their cache; the others end as
+    in a normal call, and so does every later call."""
+    rng = np.random.default_rng(V)
+    T, cap, mp = 8, 64, 6
+    tl = np.array([1, 4, 0, 8], np.int32)
+    made = [1, 4, 0, mp + 1]  # such exchanges; the third is malformed, the last cut by max_path
+    B = len(tl)
+    par = np.full((B, T), -1, np.int32)
+    for b in range(B):
+        par[b, 1:tl[b]] = [0, 0, 2, 3, 4, 5, 6][:max(0, int(tl[b]) - 1)]
+    f = lambda a: torch.as_tensor(a).cuda()  # noqa: E731
+    tgt = (2 * torch.randn((B, T, V), generator=torch.Generator().manual_seed(1))).to(dtype).cuda()
+    drf = tgt.clone()
+    tok = np.stack([rng.permutation(V)[:T] for _ in range(B)]).astype(np.int32)
+    for b in range(B):  # the root's children: the draft says too much of node 1, too little of node 2
+        drf[b, 0, tok[b, 1]] += 8
+        drf[b, 0, tok[b, 2]] -= 5
+    tree = dreams.Tree(f(par), f(tok), f(tl), f(np.array([9, 50, 3, 20], np.int32)))
+    bits = torch.from_numpy(rng.integers(-32768, 32768, (2, 3, B, cap, 2, 64)).astype(np.int16)).cuda()
+    ua, ur = torch.zeros((B, T), device="cuda"), torch.rand((B, T), device="cuda")
+    ua[:, 1] = 0.5
+
+    def run():
+        k, v = bits[0].clone(), bits[1].clone()
+        kv = dreams.KVCache(k.view(torch.bfloat16), v.view(torch.bfloat16))
+        outs = tuple(torch.full(s, -5, dtype=torch.int32, device="cuda") for s in ((B,), (B, mp), (B, mp), (B,)))
+        st = torch.zeros(1, dtype=torch.int32, device="cuda")
+        dreams.verify_step_speculative(tgt, drf, tree, kv, mp, 1.0, ua, ur, outputs=outs, status=st)
+        torch.cuda.synchronize()
+        return [*outs, k.transpose(0, 1), v.transpose(0, 1)], int(st.item())
+
+    untouched = [torch.full_like(t, -5) for t in run()[0][:4]] + [bits[0].transpose(0, 1), bits[1].transpose(0, 1)]
+    ref, st = run()
+    assert st == dreams.DATA_BAD_TREE_LEN
+    assert ref[0].tolist() == [1, 3, 0, mp] and not torch.equal(ref[4], untouched[4])
+    for x in (0, 1, 3, 4, mp, mp + 1, 500):
+        try:
+            dreams.test_set_stall(dreams.TEST_SPECULATIVE, x, 20_000_000)
+            got, st = run()
+        finally:
+            dreams.test_set_stall(0, -1)
+        assert st == dreams.DATA_BAD_TREE_LEN | (dreams.DATA_TIMEOUT if x < max(made) else 0), x
+        for b in range(B):
+            want = untouched if x < made[b] else ref
+            for a, w in zip(got, want):
+                assert torch.equal(a[b], w[b]), (x, b)
+        again, st = run()
+        assert st == dreams.DATA_BAD_TREE_LEN and all(torch.equal(a, w) for a, w in zip(again, ref))
