@@ -14,6 +14,10 @@ equal its own greedy prediction; here the drafts form a tree.
 
     out, lse = tree_verify_attn(q, kv, tree, scale)          # per layer
     res = verify_step(logits, tree, kv, max_path)            # argmax + walk + compaction
+
+With ``stream=`` a call runs on that stream, as does the zero-fill of the
+workspace kept for it. Outputs that the call creates belong to the current
+stream; a caller with several streams hands in its own, or orders the two.
 """
 from __future__ import annotations
 
@@ -189,7 +193,8 @@ def _call_ws(name: str, dev: torch.device, kind: str, size, workspace: Optional[
         ptr, nbytes = (None, 0) if ws is None else (ws.data_ptr(), ws.numel())
         st = _status_of(name, dev, (*head, ptr, nbytes, *tail, handle))
         if st == ERR_WORKSPACE:
-            ws = _WS[key] = torch.zeros(size(), dtype=torch.uint8, device=dev)
+            with torch.cuda.stream(stream):  # (None: the current one)
+                ws = _WS[key] = torch.zeros(size(), dtype=torch.uint8, device=dev)
             st = _status_of(name, dev, (*head, ws.data_ptr(), ws.numel(), *tail, handle))
     _check(name, st)
 
