@@ -1356,22 +1356,17 @@ __device__ __forceinline__ bool spec_cluster_ms(SpecShared &sh, const SpecParams
   return true;
 }
 
-// Warp 0: the parent and token rows of a sequence into sh (entries past
-// tree_len: parent -1, token 0); DREAMS_DATA_BAD_PARENT when parent[0] != -1
-// or a parent[i] lies outside [0, i). pre_par / pre_tok: the rows' first Tm
-// entries, loaded before tree_len was known.
-__device__ int spec_tree_warp(SpecShared &sh, const int (&pre_par)[2], const int (&pre_tok)[2], int T) {
-  const int lane = threadIdx.x & 31;
+// DREAMS_DATA_* of a sequence's lengths and parent row (0: valid), one warp;
+// par: the entries 32 h + lane of the row, loaded before tree_len was known.
+__device__ __forceinline__ int spec_check(const SpecParams &p, int TL, int L, const int (&par)[2]) {
+  if (TL < 1 || TL > p.tr.T_max) return DREAMS_DATA_BAD_TREE_LEN;
+  if (L < 0 || L > p.kv.capacity - TL) return DREAMS_DATA_BAD_KV_LEN;
   int bad = 0;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    const int i = lane + 32 * h;
-    const bool live = i < T;
-    const int pa = live ? pre_par[h] : -1;
-    sh.par[i] = pa;
-    sh.tok[i] = live ? pre_tok[h] : 0;
-    if (i == 0) bad |= pa != -1;
-    else if (live) bad |= pa < 0 || pa >= i;
+    const int i = int(threadIdx.x & 31) + 32 * h;
+    if (i == 0) bad |= par[h] != -1;
+    else if (i < TL) bad |= par[h] < 0 || par[h] >= i;
   }
   return __any_sync(0xffffffffu, bad) ? DREAMS_DATA_BAD_PARENT : 0;
 }
@@ -1571,8 +1566,8 @@ __device__ int spec_slice_draw(SpecShared &sh, const float *et, const float *ed,
 // One cluster of p.cs CTAs per sequence (grid.x = B * cs): the walk with its
 // decisions, the bonus draw, the outputs and the KV compaction. A chain of
 // dependent steps, so its latency is what counts: 16 trees of 32-64 nodes at
-// 128256 bf16 entries took 47.8 us a pass, 31.9 with the root's rows loaded
-// under the tree check, exponentials from registers, conflict-free slices, warp
+// 128256 bf16 entries took 47.8 us a pass, 32.5 with the root's rows loaded
+// while the tree is laid out, exponentials from registers, conflict-free slices, warp
 // maxima by one instruction, the outputs written by the CTA that draws, and the
 // first child's rows prefetched.
 template <typename T>
@@ -1600,30 +1595,36 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
   const int64_t v0 = int64_t(rank) * S;
   float *et = spec_dyn, *ed = spec_dyn + S;
   const float k2 = p.k2;
-  // the tree rows go out with the lengths (rows of T_max entries exist)
-  int pre_par[2] = {-1, -1}, pre_tok[2] = {0, 0};
-  if (warp == 0) {
+  // the tree rows go out with the lengths (rows of T_max entries exist); every
+  // warp checks the tree for itself
+  int par[2] = {-1, -1}, tok[2] = {0, 0};
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int i = lane + 32 * h;
-      if (i < Tm) {
-        pre_par[h] = ld_issue_now(p.tr.parent + rb + i);
-        pre_tok[h] = ld_issue_now(p.tr.tokens + rb + i);
-      }
+  for (int h = 0; h < 2; ++h) {
+    const int i = lane + 32 * h;
+    if (i < Tm) {
+      par[h] = ld_issue_now(p.tr.parent + rb + i);
+      if (warp == 0) tok[h] = ld_issue_now(p.tr.tokens + rb + i);
     }
   }
   const int TL = ld_issue_now(p.tr.tree_len + b), L = ld_issue_now(p.tr.kv_len + b);
-  // the root's rows (bf16: both; f32: the target's) are on their way while the
-  // tree is checked
+  const int bad = spec_check(p, TL, L, par);
+  // the root's rows (bf16: both; f32: the target's) are on their way while warp
+  // 0 lays out the tree; a row is read only where the walk visits its node, the
+  // draft's only where it tries a child (a valid tree's node 1 is the root's)
   constexpr bool PAIR = sizeof(T) == 2;  // both rows' words fit in registers
   uint4 wt[SPEC_MAX_J][sizeof(T) / 2], wd[PAIR ? SPEC_MAX_J : 1][PAIR ? sizeof(T) / 2 : 1];
-  spec_issue<T>(p, static_cast<const T *>(p.tgt) + rb * p.row_stride, v0, wt);
-  if constexpr (PAIR) spec_issue<T>(p, static_cast<const T *>(p.drf) + rb * p.row_stride, v0, wd);
+  if (!bad) {
+    spec_issue<T>(p, static_cast<const T *>(p.tgt) + rb * p.row_stride, v0, wt);
+    if constexpr (PAIR)
+      if (TL > 1 && p.max_path > 1) spec_issue<T>(p, static_cast<const T *>(p.drf) + rb * p.row_stride, v0, wd);
+  }
   if (warp == 0) {
-    int bad = 0;
-    if (TL < 1 || TL > Tm) bad = DREAMS_DATA_BAD_TREE_LEN;
-    else if (L < 0 || L > p.kv.capacity - TL) bad = DREAMS_DATA_BAD_KV_LEN;
-    else bad = spec_tree_warp(sh, pre_par, pre_tok, TL);
+    // entries past tree_len: parent -1, token 0
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      sh.par[lane + 32 * h] = lane + 32 * h < TL ? par[h] : -1;
+      sh.tok[lane + 32 * h] = lane + 32 * h < TL ? tok[h] : 0;
+    }
     // the entries of the pages that hold the tree's slots, for the compaction
     if (lane < 2) {
       const int pg = (L >> 6) + lane;
@@ -1631,14 +1632,10 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
                         ? __ldg(p.kv.page_table + int64_t(b) * p.kv.pages_per_seq + pg)
                         : -1;
     }
-    if (lane == 0) {
-      sh.cmd = bad;
-      if (bad && rank == 0) flag(p.status, bad);
-    }
+    if (lane == 0 && bad && rank == 0) flag(p.status, bad);
   }
   __syncthreads();
   cluster_wait();
-  const bool bad = sh.cmd != 0;
   int n = -1, bonus = 0, xc = 0;  // xc: exchanges that have arrived
   bool dead = false;              // one did not
   bool sent = false, agreed = false;  // arrived at the cluster's last barrier; past it

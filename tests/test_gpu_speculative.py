@@ -450,3 +450,32 @@ def test_speculative_many_exchanges(dreams, dtype, B, V):
     for r in [dreams.verify_step_speculative(tgt_t, drf_t, tree, kv, 6, tau, ua, ur, status=st) for _ in range(20)]:
         _compare(r, ref)
     assert int(st.item()) == 0
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("max_path", [1, 4])
+def test_unvisited_rows_do_not_matter(dreams, dtype, max_path):
+    """Rows that the walk has no use for hold NaN: both rows of malformed
+    sequences, the draft's of roots without children and of nodes where
+    max_path ends the walk. The results are those of finite rows there."""
+    rng = np.random.default_rng(12)
+    T, V = 6, 5000
+    tl = np.array([1, 6, 0, 6, 7, 3], np.int32)  # 2, 4: bad lengths; 3: a bad parent; 5: too long for the cache
+    kl = np.array([5, 7, 5, 5, 5, 62], np.int32)
+    B = len(tl)
+    par = np.full((B, T), -1, np.int32)
+    par[[1, 3], 1:] = np.arange(T - 1)
+    par[3, 2] = 2
+    par[5, 1:3] = 0
+    tgt = (2 * torch.randn((B, T, V), generator=torch.Generator().manual_seed(3))).to(dtype).cuda()
+    drf = tgt.clone()
+    tok, u = rng.integers(0, V, (B, T)).astype(np.int32), np.zeros((B, T), np.float32)
+    u_res = rng.random((B, T), dtype=np.float32)
+    k = torch.zeros((B, 64, 1, 64), dtype=torch.bfloat16, device="cuda")
+    ref, st = _run(dreams, tgt, drf, par, tok, tl, kl, k, k.clone(), max_path, 1.0, u, u_res)
+    bad = dreams.DATA_BAD_TREE_LEN | dreams.DATA_BAD_PARENT | dreams.DATA_BAD_KV_LEN
+    assert st == bad and ref["accept_len"].tolist() == [1, max_path, 0, 0, 0, 0]
+    tgt[2:], drf[2:], drf[0] = float("nan"), float("nan"), float("nan")
+    drf[1, max_path - 1:], tgt[1, max_path:], tgt[0, 1:] = float("nan"), float("nan"), float("nan")
+    got, st = _run(dreams, tgt, drf, par, tok, tl, kl, k, k.clone(), max_path, 1.0, u, u_res)
+    assert st == bad and all(torch.equal(got[key], ref[key]) for key in ref)
