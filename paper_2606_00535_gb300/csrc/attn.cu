@@ -124,14 +124,6 @@ constexpr int ATTN_CAUSAL = 2;  // slots 0 .. kv_len + t for query t (prefill se
 // causal), or the prefix alone (full).
 __device__ __forceinline__ int key_total(const AttnParams &p, int L, int T) { return p.mode == ATTN_FULL ? L : L + T; }
 
-// A read-only global load issued where it stands (the compiler may not sink it
-// to the value's first use).
-__device__ __forceinline__ int ld_issue_now(const int32_t *ptr) {
-  int v;
-  asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(v) : "l"(ptr));
-  return v;
-}
-
 struct TcParams {
   CUtensorMap tmap_q;
   CUtensorMap tmap_k;

@@ -53,6 +53,9 @@ inline dreams_status_t check_launch() {
 // A kernel that reads global memory before its wait may read only what its own
 // predecessor's inputs were (the walk's tree arrays), and reads it through L2
 // (__ldcg): L1 may hold older lines until the wait.
+// cluster: the CTAs of a cluster; 0 for a kernel without clusters. (A cluster of
+// one CTA needs the attribute too: without it the walk's st.async faulted as an
+// illegal instruction.)
 template <typename... Params, typename... Args>
 dreams_status_t launch_clusters(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                                 int cluster, Args... args) {
@@ -69,7 +72,7 @@ dreams_status_t launch_clusters(void (*kernel)(Params...), dim3 grid, dim3 block
   attr[1].val.clusterDim.y = 1;
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  cfg.numAttrs = cluster > 0 ? 2 : 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
   if (e != cudaSuccess) {
     set_last_cuda_error(e);
@@ -81,7 +84,7 @@ dreams_status_t launch_clusters(void (*kernel)(Params...), dim3 grid, dim3 block
 template <typename... Params, typename... Args>
 dreams_status_t launch_kernel(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                               Args... args) {
-  return launch_clusters(kernel, grid, block, smem, stream, 1, args...);
+  return launch_clusters(kernel, grid, block, smem, stream, 0, args...);
 }
 
 // Waits until the preceding grid has completed and its writes are visible.
@@ -112,6 +115,14 @@ __device__ __forceinline__ uint32_t cluster_addr(const void *local_ptr, uint32_t
   return ra;
 }
 
+// A read-only global load issued where it stands (the compiler may not sink it
+// to the value's first use), so that its latency overlaps the work in between.
+__device__ __forceinline__ int ld_issue_now(const int32_t *ptr) {
+  int v;
+  asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(v) : "l"(ptr));
+  return v;
+}
+
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 __device__ __forceinline__ void flag(int32_t *status_word, int32_t bits) {
@@ -127,7 +138,6 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// 16-byte global -> shared copy; src_bytes == 0 zero-fills the destination.
 // Order-preserving integer key of an f32 bit pattern for the argmax order:
 // greater value -> greater key, +0 == -0, NaN above every number.
 __device__ __forceinline__ int order_key(uint32_t u) {

@@ -57,12 +57,6 @@ __device__ __forceinline__ float fmax_nan(float a, float b) {
   asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
   return d;
 }
-// 2^x by the hardware approximation (ex2.approx, subnormals flushed to zero).
-__device__ __forceinline__ float exp2f_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 
 template <typename T>
 struct Elem;
@@ -104,52 +98,49 @@ __device__ void block_argmax(const T *row, int64_t begin, int64_t end, bool vec_
   constexpr int VEC = E::VEC;
   const int tid = threadIdx.x;
   int bk = INT_MIN, bi = INT_MAX;
-  int64_t vend = begin;
-  {
-    // a chunk that does not start on 16 bytes: the values before the first
-    // boundary one by one, then vectors like any other (854 x 128257 bf16: 35
-    // us; value by value the whole row took 103)
-    if (!vec_ok) {
-      const int64_t head =
-          std::min<int64_t>(end, begin + int((16 - (reinterpret_cast<uintptr_t>(row + begin) & 15)) & 15) / int(sizeof(T)));
-      if (begin + tid < head) {
-        bk = order_key(E::bits(row, begin + tid));
-        bi = int(begin + tid);
-      }
-      begin = head;
+  // a chunk that does not start on 16 bytes: the values before the first
+  // boundary one by one, then vectors like any other (854 x 128257 bf16: 35
+  // us; value by value the whole row took 103)
+  if (!vec_ok) {
+    const int64_t head =
+        std::min<int64_t>(end, begin + int((16 - (reinterpret_cast<uintptr_t>(row + begin) & 15)) & 15) / int(sizeof(T)));
+    if (begin + tid < head) {
+      bk = order_key(E::bits(row, begin + tid));
+      bi = int(begin + tid);
     }
-    const int64_t nvec = (end - begin) / VEC;
-    vend = begin + nvec * VEC;
-    const uint4 *vp = reinterpret_cast<const uint4 *>(row + begin);
-    int64_t best_v = -1;
-    int64_t vi = tid;
-    constexpr int U = 4;
-    for (; vi + (U - 1) * ARGMAX_THREADS < nvec; vi += U * ARGMAX_THREADS) {
-      uint4 x[U];
+    begin = head;
+  }
+  const int64_t nvec = (end - begin) / VEC;
+  const int64_t vend = begin + nvec * VEC;
+  const uint4 *vp = reinterpret_cast<const uint4 *>(row + begin);
+  int64_t best_v = -1;
+  int64_t vi = tid;
+  constexpr int U = 4;
+  for (; vi + (U - 1) * ARGMAX_THREADS < nvec; vi += U * ARGMAX_THREADS) {
+    uint4 x[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) x[u] = __ldcs(vp + vi + u * ARGMAX_THREADS);
+    for (int u = 0; u < U; ++u) x[u] = __ldcs(vp + vi + u * ARGMAX_THREADS);
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int k = E::vec_key(x[u]);
-        if (k > bk) {
-          bk = k;
-          best_v = vi + u * ARGMAX_THREADS;
-        }
-      }
-    }
-    for (; vi < nvec; vi += ARGMAX_THREADS) {
-      const int k = E::vec_key(__ldcs(vp + vi));
+    for (int u = 0; u < U; ++u) {
+      const int k = E::vec_key(x[u]);
       if (k > bk) {
         bk = k;
-        best_v = vi;
+        best_v = vi + u * ARGMAX_THREADS;
       }
     }
-    if (best_v >= 0) {  // (a later vector's key is greater than any value's before it)
-      const uint4 x = __ldg(vp + best_v);
-#pragma unroll
-      for (int j = VEC - 1; j >= 0; --j)
-        if (order_key(E::lane_bits(x, j)) == bk) bi = int(begin + best_v * VEC + j);
+  }
+  for (; vi < nvec; vi += ARGMAX_THREADS) {
+    const int k = E::vec_key(__ldcs(vp + vi));
+    if (k > bk) {
+      bk = k;
+      best_v = vi;
     }
+  }
+  if (best_v >= 0) {  // (a later vector's key is greater than any value's before it)
+    const uint4 x = __ldg(vp + best_v);
+#pragma unroll
+    for (int j = VEC - 1; j >= 0; --j)
+      if (order_key(E::lane_bits(x, j)) == bk) bi = int(begin + best_v * VEC + j);
   }
   for (int64_t i = vend + tid; i < end; i += ARGMAX_THREADS) {
     const int k = order_key(E::bits(row, i));
@@ -367,10 +358,10 @@ __device__ __forceinline__ float words_sum(const uint4 *w, int n, bool bf16, flo
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       if (bf16) {
-        s += exp2f_approx((__uint_as_float(v[i] << 16) - m) * k2);
-        s += exp2f_approx((__uint_as_float(v[i] & 0xffff0000u) - m) * k2);
+        s += tc::ex2((__uint_as_float(v[i] << 16) - m) * k2);
+        s += tc::ex2((__uint_as_float(v[i] & 0xffff0000u) - m) * k2);
       } else {
-        s += exp2f_approx((__uint_as_float(v[i]) - m) * k2);
+        s += tc::ex2((__uint_as_float(v[i]) - m) * k2);
       }
     }
   }
@@ -466,10 +457,10 @@ __device__ int sample_select_warp(const SampleParams &p, const T *row, const flo
         first_inf = min(first_inf, g);
       } else if (v[i].x != -INFINITY) {
         if (v[i].x > m_l) {
-          z_l = (m_l == -INFINITY ? 0.f : z_l * exp2f_approx((m_l - v[i].x) * k2)) + v[i].y;
+          z_l = (m_l == -INFINITY ? 0.f : z_l * tc::ex2((m_l - v[i].x) * k2)) + v[i].y;
           m_l = v[i].x;
         } else {
-          z_l += v[i].y * exp2f_approx((v[i].x - m_l) * k2);
+          z_l += v[i].y * tc::ex2((v[i].x - m_l) * k2);
         }
       }
     }
@@ -504,7 +495,7 @@ __device__ int sample_select_warp(const SampleParams &p, const T *row, const flo
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
   if (M == -INFINITY) return 0;  // every value -inf: the argmax is index 0
-  float Z = m_l == -INFINITY ? 0.f : z_l * exp2f_approx((m_l - M) * k2);
+  float Z = m_l == -INFINITY ? 0.f : z_l * tc::ex2((m_l - M) * k2);
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, off);
   const float uc = u > 0.f ? fminf(u, 1.f) : 0.f;  // NaN and negatives count as 0
@@ -525,7 +516,7 @@ __device__ int sample_select_warp(const SampleParams &p, const T *row, const flo
     int llast = -1;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      c[i] = v[i].x != -INFINITY ? v[i].y * exp2f_approx((v[i].x - M) * k2) : 0.f;
+      c[i] = v[i].x != -INFINITY ? v[i].y * tc::ex2((v[i].x - M) * k2) : 0.f;
       ls += c[i];
       if (c[i] > 0.f) llast = base + 8 * lane + i;
     }
@@ -551,7 +542,7 @@ __device__ int sample_select_warp(const SampleParams &p, const T *row, const flo
           if (g_hit < 0 && c[i] > 0.f) {
             if (acc + c[i] > t) {
               g_hit = base + 8 * lane + i;
-              r_hit = fmaxf(t - acc, 0.f) / exp2f_approx((v[i].x - M) * k2);  // >= 0: positive weight
+              r_hit = fmaxf(t - acc, 0.f) / tc::ex2((v[i].x - M) * k2);  // >= 0: positive weight
             } else {
               g_prev = base + 8 * lane + i;
             }
@@ -596,7 +587,7 @@ __device__ int sample_select_warp(const SampleParams &p, const T *row, const flo
     float w[8], ls = 0.f;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      w[i] = exp2f_approx((x[i] - m) * k2);
+      w[i] = tc::ex2((x[i] - m) * k2);
       ls += w[i];
     }
     float linc = ls;
@@ -1219,13 +1210,7 @@ struct SpecShared {
   int32_t cmd;
 };
 
-// Loads issued where they stand (volatile), so that their latency overlaps the
-// work between the load and the first use of its value.
-__device__ __forceinline__ int ld_issue_now(const int32_t *ptr) {
-  int v;
-  asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(v) : "l"(ptr));
-  return v;
-}
+// ld_issue_now for other types.
 __device__ __forceinline__ float ld_now_f32(const float *ptr) {
   float v;
   asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(ptr));
@@ -1261,8 +1246,8 @@ __device__ __forceinline__ float warp_max(float v) {
 // from each lane's pair (x, y) and (z, w); lane 0's bits on every lane.
 __device__ __forceinline__ float4 ms4_lanes(float4 v, float k2) {
   const float Mt = warp_max(v.x), Md = warp_max(v.z);
-  const float st = v.x == -INFINITY ? 0.f : v.y * exp2f_approx((v.x - Mt) * k2);
-  const float sd = v.z == -INFINITY ? 0.f : v.w * exp2f_approx((v.z - Md) * k2);
+  const float st = v.x == -INFINITY ? 0.f : v.y * tc::ex2((v.x - Mt) * k2);
+  const float sd = v.z == -INFINITY ? 0.f : v.w * tc::ex2((v.z - Md) * k2);
   return make_float4(Mt, warp_sum_bcast(st), Md, warp_sum_bcast(sd));
 }
 
@@ -1426,10 +1411,10 @@ __device__ __forceinline__ float2 spec_exps(const SpecParams &p, const uint4 (&w
       for (int h = 0; h < 2; ++h) {
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);  // (every value past V)
         if (m != -INFINITY) {
-          v.x = exp2f_approx((value(j, 4 * h) - m) * p.k2);
-          v.y = exp2f_approx((value(j, 4 * h + 1) - m) * p.k2);
-          v.z = exp2f_approx((value(j, 4 * h + 2) - m) * p.k2);
-          v.w = exp2f_approx((value(j, 4 * h + 3) - m) * p.k2);
+          v.x = tc::ex2((value(j, 4 * h) - m) * p.k2);
+          v.y = tc::ex2((value(j, 4 * h + 1) - m) * p.k2);
+          v.z = tc::ex2((value(j, 4 * h + 2) - m) * p.k2);
+          v.w = tc::ex2((value(j, 4 * h + 3) - m) * p.k2);
         }
         *reinterpret_cast<float4 *>(e + spec_at(j, h)) = v;
         s0 += v.x + v.y;
@@ -1697,14 +1682,14 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
       const float Mt = g.x, Zd = g.w;
       // this thread's factors to the rows' maxima (its exponentials are
       // relative to its own maxima), and their ratio for the passes
-      const float at = m.x == -INFINITY ? 0.f : exp2f_approx((m.x - Mt) * k2);
-      const float ad = m.y == -INFINITY ? 0.f : exp2f_approx((m.y - g.z) * k2);
+      const float at = m.x == -INFINITY ? 0.f : tc::ex2((m.x - Mt) * k2);
+      const float ad = m.y == -INFINITY ? 0.f : tc::ex2((m.y - g.z) * k2);
       const float rd = at > 0.f ? ad / at : 0.f;
       float c = 0.f, Pu = g.y;  // the residual ~ max(0, et - c ed), Pu its sum
       int next = -1;
       for (uint64_t rest = try_kids ? kids : 0; rest != 0; rest &= rest - 1) {
         const int ch = __ffsll(static_cast<long long>(rest)) - 1;
-        const float et_x = exp2f_approx((sh.cxt[ch] - Mt) * k2), ed_x = exp2f_approx((sh.cxd[ch] - g.z) * k2);
+        const float et_x = tc::ex2((sh.cxt[ch] - Mt) * k2), ed_x = tc::ex2((sh.cxd[ch] - g.z) * k2);
         const float num = fmaxf(fmaf(-c, ed_x, et_x), 0.f);
         float a = 0.f;  // min(1, r(x) / q(x)) = Zd num / (Pu ed_x); q(x) = 0: 1 when r(x) > 0
         if (num > 0.f) a = ed_x > 0.f ? fminf(1.f, (num / ed_x) * (Zd / Pu)) : 1.f;
@@ -2208,26 +2193,8 @@ extern "C" dreams_status_t dreams_verify_step_speculative(
       return DREAMS_ERR_CUDA;
     }
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned(int64_t(tree->B) * pl.cs));
-  cfg.blockDim = dim3(SPEC_THREADS);
-  cfg.dynamicSmemBytes = size_t(smem);
-  cfg.stream = reinterpret_cast<cudaStream_t>(stream);
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = unsigned(pl.cs);
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, p);
-  if (e != cudaSuccess) {
-    set_last_cuda_error(e);
-    return DREAMS_ERR_CUDA;
-  }
-  return check_launch();
+  return launch_clusters(kernel, dim3(unsigned(int64_t(tree->B) * pl.cs)), dim3(SPEC_THREADS), size_t(smem),
+                         reinterpret_cast<cudaStream_t>(stream), pl.cs, p);
 }
 
 // ------------------------------------------------------------------ no-allocation argmax
