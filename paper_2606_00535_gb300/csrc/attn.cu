@@ -247,9 +247,15 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_c
   constexpr uint32_t KV_TILE = NR * KV_REGION;   // one K or V tile
   constexpr uint32_t IDESC_QK = tc::idesc_bf16_f32(ROWS, KT, false);
   constexpr uint32_t IDESC_PV = tc::idesc_bf16_f32(ROWS, D, true);
-  // keys of a tile's first P hand-off: with the entropy sums the softmax is
-  // longer and 96 did better (prefill of 3392 tokens x 32 heads 103.2 against
-  // 106.5 us), without them 64 (3392 slots x 32 heads 18.0 against 18.3 us)
+  // Keys of a tile's first P hand-off. Without the entropy sums 64 against 96
+  // keys, us of GPU time at D = 128 | 64: causal prefill of 3392 tokens x 32
+  // heads 93.4 / 96.6 | 78.5 / 79.5, of 1500 31.5 / 33.0 | 26.0 / 26.7, of 500
+  // 10.3 / 10.4 | 8.9 / 9.0; one tree on 3392 slots x 32 heads 18.5 / 19.2 | 14.4
+  // / 14.4; 16 paged trees of 1500-6000 slots x 8 heads 55.5 / 56.8 | 46.8 / 47.1;
+  // cross-attention to 3392 slots 17.9 / 18.8 | 13.0 / 13.0. The entropy sums
+  // make the softmax longer, and 96 is the better one: prefill of 3392 tokens
+  // 106.9 / 104.1 | 91.0 / 89.4, of 1500 35.4 / 34.9 | 29.4 / 29.0, of 500 11.0 /
+  // 11.0 | 9.6 / 9.6.
   constexpr int FIRST = ENT ? 96 : 64;
 
   extern __shared__ uint8_t smem_raw[];
@@ -606,9 +612,8 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_c
       const uint64_t qd0 = tc::smem_desc_sw128(q_s, 16, 1024);
       const uint64_t kd0 = tc::smem_desc_sw128(k_s(0), 16, 1024);
       const uint64_t vd0 = tc::smem_desc_sw128(v_s(0), KV_REGION, 1024);
-      // The MMAs are issued by the converged warp, so that their operands stay
-      // in uniform registers (tc.cuh): batched serving (16 sequences, 32 q / 8
-      // KV heads, 1500-6000 slots) 77.5 -> 70.0 us a pass, the causal prefill
+      // The MMAs are issued by the converged warp, which issues them faster than
+      // one lane does (tc.cuh): batched serving (16 sequences, 32 q / 8 KV heads, 1500-6000 slots) 77.5 -> 70.0 us a pass, the causal prefill
       // of 3392 tokens x 32 heads 122.9 -> 118.8 us. Waits for P, V and K then
       // hide under the MMAs that are queued: the softmax warps, whose chain of
       // scores, exponents and hand-off bounds a tile, wait for no copy (64.8

@@ -7,8 +7,8 @@
 // tcgen05 GEMM, persistent, on pairs of CTAs (cta_group::2, two SMs). A tile is
 // 256 vocabulary entries (the MMA's M side, 128 per CTA) by up to 256 rows of H
 // (its N side, of which each CTA loads half), so that a 64-column block of the
-// largest tile costs each SM 32 KB from L2, where a CTA by itself reads 48 KB
-// for half the work, and few rows cost no padding to 128. 320 threads per CTA:
+// largest tile costs each SM 32 KB from L2 for its 128 x 256 share, where a CTA
+// by itself reads 48 KB, and few rows cost no padding to 128. 320 threads per CTA:
 //   warp 0, one thread  TMA producer: this CTA's halves of W and H, two blocks
 //                       of 64 columns (128-byte swizzle) per ring stage
 //   warp 1, converged   in the even CTA the MMA issuer (M256 K16, bf16 -> f32)

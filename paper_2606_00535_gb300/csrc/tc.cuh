@@ -174,12 +174,11 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t *r) {
 
 // ---------------------------------------------------------------- MMA
 // The MMA wrappers are called by a whole converged warp; `leader` (elect_one)
-// is non-zero in the one lane whose instruction takes effect. The operands
-// (descriptors, TMEM addresses) sit in uniform registers: with the warp
-// converged the compiler keeps them there, while in a one-lane branch it moves
-// them from vector registers for every MMA, which measured about 93 clk per
-// MMA inside the attention kernel instead of 26-37 (an M128 N128 K16 MMA takes
-// 64 on the tensor pipe).
+// is non-zero in the one lane whose instruction takes effect. Issued from a
+// one-lane branch an MMA took about 93 clk inside the attention kernel instead
+// of 26-37 (an M128 N128 K16 MMA takes 64 on the tensor pipe); the likely reason
+// is that the operands (descriptors, TMEM addresses) are wanted in uniform
+// registers, which a converged warp can compute them in.
 __device__ __forceinline__ uint32_t elect_one() {
   uint32_t r;
   asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
