@@ -613,9 +613,10 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_tc_kernel(const __grid_c
       const uint64_t kd0 = tc::smem_desc_sw128(k_s(0), 16, 1024);
       const uint64_t vd0 = tc::smem_desc_sw128(v_s(0), KV_REGION, 1024);
       // The MMAs are issued by the converged warp, which issues them faster than
-      // one lane does (tc.cuh): batched serving (16 sequences, 32 q / 8 KV heads, 1500-6000 slots) 77.5 -> 70.0 us a pass, the causal prefill
-      // of 3392 tokens x 32 heads 122.9 -> 118.8 us. Waits for P, V and K then
-      // hide under the MMAs that are queued: the softmax warps, whose chain of
+      // one lane does (tc.cuh): batched serving (16 sequences, 32 q / 8 KV heads,
+      // 1500-6000 slots) 77.5 -> 70.0 us a pass, the causal prefill of 3392
+      // tokens x 32 heads 122.9 -> 118.8 us. Waits for P, V and K then hide
+      // under the MMAs that are queued: the softmax warps, whose chain of
       // scores, exponents and hand-off bounds a tile, wait for no copy (64.8
       // -> 62.6 and 109.8 -> 104.2 us of GPU time against a softmax thread
       // that saw the copies land before it handed P over).
