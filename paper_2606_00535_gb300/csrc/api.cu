@@ -87,7 +87,8 @@ extern "C" dreams_status_t dreams_test_set_stall(int32_t kernels, int32_t stall_
     dreams::g_stall_wait_ns.store(dreams::DEFAULT_WAIT_NS);
     return DREAMS_OK;
   }
-  if ((kernels & ~(DREAMS_TEST_ATTENTION | DREAMS_TEST_LM_HEAD | DREAMS_TEST_SPECULATIVE)) != 0 || kernels == 0 || wait_limit_ns < 1000 ||
+  const int32_t known = DREAMS_TEST_ATTENTION | DREAMS_TEST_LM_HEAD | DREAMS_TEST_SPECULATIVE;
+  if ((kernels & ~known) != 0 || kernels == 0 || wait_limit_ns < 1000 ||
       wait_limit_ns > int64_t(dreams::DEFAULT_WAIT_NS))
     return DREAMS_ERR_INVALID_ARG;
   dreams::g_stall_wait_ns.store(uint64_t(wait_limit_ns));
