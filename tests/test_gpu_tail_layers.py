@@ -76,7 +76,7 @@ def test_tail_compacts_every_layer(dreams, layers, Hkv, D, paged, own_pred):
 
 
 @pytest.mark.parametrize("layers,B,T,V", [(32, 16, 64, 600), (4, 3, 9, 5000)])
-@pytest.mark.parametrize("call", ["greedy", "greedy_own", "sampled"])
+@pytest.mark.parametrize("call", ["greedy", "greedy_own", "sampled", "speculative"])
 def test_lengths_advance_in_place(dreams, call, layers, B, T, V):
     """Calls in a row on one cache, each on the lengths that the call before
     wrote over its own. With 32 layers, 16 sequences and 64 rows each, 512 CTAs
@@ -95,7 +95,8 @@ def test_lengths_advance_in_place(dreams, call, layers, B, T, V):
     for b in range(B):  # every node's first child is its prediction
         for i in range(int(tl[b]) - 1, 0, -1):
             x[b, par[b, i], tok[b, i]] = 50.0 + (int(tl[b]) - i)
-    logits, u = f(x), f(rng.random((B, T), dtype=np.float32))
+    u_np, zero = rng.random((B, T), dtype=np.float32), np.zeros((B, T), np.float32)
+    logits, u, u0 = f(x), f(u_np), f(zero)
     pred = oracle.argmax(x.reshape(-1, V)).reshape(B, T)
     lay = oracle.KVLayout(cap, Hkv, D)
     ko, vo = (rng.integers(0, 1 << 16, (layers, B, cap, Hkv, D), np.uint16) for _ in range(2))
@@ -108,13 +109,16 @@ def test_lengths_advance_in_place(dreams, call, layers, B, T, V):
         out = (acc, path, toks, tree.kv_len)
         if call == "sampled":  # at this temperature the draws are the argmax
             dreams.verify_step_sampled(logits, tree, kv, 4, 1e-3, u, outputs=out, status=st)
+        elif call == "speculative":  # draft == target and uniforms of 0: first children are accepted
+            dreams.verify_step_speculative(logits, logits, tree, kv, 4, 1e-3, u0, u, outputs=out, status=st)
         else:
             dreams.verify_step(logits, tree, kv, 4, argmax_out=am, outputs=out, status=st)
     torch.cuda.synchronize()
     assert int(st.item()) == 0
     kl = kl0
     for _ in range(steps):
-        ref = oracle.accept_path(pred, par, tok, tl, kl, 4)
+        ref = (oracle.spec_path(x, x, par, tok, tl, kl, 4, 1e-3, zero, u_np) if call == "speculative" else
+               oracle.accept_path(pred, par, tok, tl, kl, 4))
         for n in range(layers):
             ko[n], vo[n], ost = oracle.kv_compact(ko[n], vo[n], lay, kl, ref["accept_len"], ref["path"])
             assert ost == 0
