@@ -46,3 +46,10 @@ def test_unaligned_rows_equal_aligned_rows(dreams, dtype, offset, V):
     am = dreams.vocab_argmax(wide).cpu().numpy()
     ref = oracle.argmax(W.bits(x), bf16_bits=True) if dtype == torch.bfloat16 else oracle.argmax(x.numpy())
     np.testing.assert_array_equal(am, ref)
+
+
+@pytest.mark.parametrize("V", [511, 512, 513, 519])
+@pytest.mark.parametrize("dtype,offset", [(torch.float32, 3), (torch.bfloat16, 0), (torch.bfloat16, 5)])
+def test_around_the_short_rows(dreams, dtype, offset, V):
+    """Up to 512 values the argmax takes such a row value by value."""
+    test_unaligned_rows_equal_aligned_rows(dreams, dtype, offset, V)
