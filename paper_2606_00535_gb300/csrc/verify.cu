@@ -1096,20 +1096,20 @@ __global__ void __launch_bounds__(TAIL_THREADS, 4) verify_tail_kernel(const Step
   // The ticket, whose round trip runs under the moves, counts the CTAs in its
   // low half. It also adds up the walk's result, so that it depends on all that
   // the CTA has read, as the outputs depend on the ticket: no fence is needed
-  // (two took 0.7 and 0.6 us; the step of a 32-layer cache takes 11.0). Four CTAs
-  // per SM (64 registers): at three, 16 sequences of 32 layers take two waves,
-  // 20.4 us instead of 17.9.
-  uint32_t ticket = 0;
-  if (p.ntail > 1 && threadIdx.x == 0)
+  // (two took 0.7 and 0.6 us; the step of a 32-layer cache takes 11.0). Where
+  // nothing moves (the walk's result does not depend on the length, so no CTA
+  // will move anything) and no prediction is cleared, the first CTA does not wait
+  // for the others. Four CTAs per SM (64 registers): at three, 16 sequences of 32
+  // layers take two waves, 20.4 us instead of 17.9.
+  const uint32_t last = uint32_t(p.ntail - 1);
+  uint32_t ticket = part == 0 ? last : ~0u;
+  if (p.ntail > 1 && threadIdx.x == 0 && (s_walk[0] > 0 || p.pred_in_ws))
     ticket = atomicAdd(p.ticket + b * p.ticket_step, 1u + (uint32_t(s_walk[0] + 2) << 16));
   const int n = s_n;
   if (n > 0)
     compact_units(p.kv, n, s_src, s_dst, part * TAIL_THREADS + int(threadIdx.x), int64_t(p.ntail) * TAIL_THREADS);
-  if (threadIdx.x >= 32) return;
-  if (p.ntail > 1) {
-    if (int(__shfl_sync(0xffffffffu, ticket, 0) & 0xffffu) != p.ntail - 1) return;
-    if (threadIdx.x == 0) p.ticket[b * p.ticket_step] = 0;
-  }
+  if (threadIdx.x >= 32 || (__shfl_sync(0xffffffffu, ticket, 0) & 0xffffu) != last) return;
+  if (p.ntail > 1 && threadIdx.x == 0) p.ticket[b * p.ticket_step] = 0;
   write_walk(b, s_walk[0], s_walk[1], p.tr.tokens + rb, p.pred + rb, s_path, p.max_path, p.accept_len, p.path,
              p.out_tokens, p.new_kv_len, s_out);
   if (p.pred_in_ws)  // leave the workspace zero-filled
@@ -1151,13 +1151,12 @@ __global__ void __launch_bounds__(TAIL_THREADS, 4) verify_tail_kernel(const Step
 // warp combines the cs values in rank order: all CTAs hold bit-identical
 // results, take the same decisions and make the same exchanges. The walk is a
 // chain of such exchanges, so their latency is its time: one store's flight
-// instead of a cluster barrier's arrival and release (four trees whose
-// root's drafts are rejected, at 128256 bf16 entries, 14.4 us against 15.8, one
-// tree of accepted ones 17.8 against 18.4). The rows' maxima and exponential sums take one such exchange of
-// (maximum, sum) pairs. An exchange that does not arrive within the limit ends
-// the walk of the whole cluster with nothing written: the CTA's warps agree on
-// it by a vote, and the CTAs by a cluster barrier before the outputs, whose
-// arrival goes ahead of the bonus draw.
+// instead of a cluster barrier's arrival and release (four trees whose root's
+// drafts are rejected, at 128256 bf16 entries, 14.4 us against 15.8, one tree of
+// accepted ones 17.2 against 18.4). The rows' maxima and exponential sums take
+// one such exchange of (maximum, sum) pairs. An exchange that does not arrive
+// within the limit ends the walk of the whole cluster with nothing written
+// (spec_late).
 constexpr int SPEC_THREADS = 512;                    // 16 warps
 constexpr int SPEC_CHUNK = 8 * SPEC_THREADS;         // values per chunk: 8 per thread
 constexpr int SPEC_MAX_J = 6;                        // chunks per CTA slice (192 KB of f32 pairs)
@@ -1273,7 +1272,7 @@ __device__ __forceinline__ void spec_send(SpecShared &sh, const SpecParams &p, f
 // warp that never voted saw the exchange arrive, so the others will too. (No
 // warp can be an exchange ahead: the next one has a barrier of the CTA before
 // its wait.)
-__device__ __noinline__ bool spec_vote(int32_t *votes, uint32_t bar, uint32_t parity) {
+__device__ __forceinline__ bool spec_vote(int32_t *votes, uint32_t bar, uint32_t parity) {
   const bool lead = (threadIdx.x & 31) == 0;
   if (lead) atomicAdd(votes, 1);
   for (;;) {
@@ -1290,27 +1289,64 @@ __device__ __noinline__ bool spec_vote(int32_t *votes, uint32_t bar, uint32_t pa
   }
 }
 
-// Waits for exchange x: true, or on every thread of the CTA false when it did
-// not arrive within the limit.
-__device__ __forceinline__ bool spec_arrived(SpecShared &sh, const SpecParams &p, int x) {
-  const uint32_t bar = smem_u32(&sh.bar[x & 1]), parity = (x >> 1) & 1;
+// Ends the threads of a CTA whose walk is given up, past the cluster's barrier:
+// flags it, and stays for the limit once more, when nothing sent to this CTA can
+// still be under way.
+__device__ __forceinline__ void spec_end(SpecShared &sh, uint32_t bar, uint32_t parity, int32_t *status,
+                                         uint64_t wait_ns) {
+  if (threadIdx.x == 0) flag(status, DREAMS_DATA_TIMEOUT);
+  tc::mbar_wait_cluster(bar, parity, &sh.zero, wait_ns);
+  asm volatile("exit;");
+}
+
+// A warp's wait for an exchange ran out. A CTA that gives the walk up tells the
+// others, meets them in a cluster barrier and ends. Without its partials none of
+// them gets past the next exchange, the bonus's at the latest, so none writes
+// anything: each of them gives up in turn. (Kept out of the walk, whose exchanges
+// take the straight path: with a result to test after each of them, and a
+// barrier before the outputs, a walk took 0.5 us more.)
+__device__ __noinline__ void spec_late(SpecShared *sh, uint32_t bar, uint32_t parity, int cs, int32_t *status,
+                                       uint64_t wait_ns) {
+  if (spec_vote(&sh->votes, bar, parity)) return;
+  if (int(threadIdx.x) < cs) st_cluster_one(&sh->dead, threadIdx.x);
+  __syncwarp();
+  cluster_sync();
+  spec_end(*sh, bar, parity, status, wait_ns);
+}
+
+// The same for the bonus's exchange. Others may have had it and be done (the
+// barrier waits for no CTA that has ended), so the CTA may give up only if one
+// gave up before; otherwise all have sent their partials, which then only have
+// to land.
+__device__ __noinline__ void spec_late_bonus(SpecShared *sh, uint32_t bar, uint32_t parity, int32_t *status,
+                                             uint64_t wait_ns) {
+  if (spec_vote(&sh->votes, bar, parity)) return;
+  __syncwarp();
+  cluster_sync();
+  if (sh->dead || !__syncthreads_and(tc::mbar_wait_cluster(bar, parity, &sh->zero, wait_ns)))
+    spec_end(*sh, bar, parity, status, wait_ns);
+}
+
+// Waits for exchange x; false when a warp's limit ran out.
+__device__ __forceinline__ bool spec_wait(uint32_t bar, uint32_t parity, uint64_t wait_ns) {
   uint64_t t0 = 0;
   for (uint32_t it = 0;; ++it) {
     if (__all_sync(0xffffffffu, tc::mbar_try_wait_cluster(bar, parity))) return true;
     if ((it & 255u) == 255u) {
       const uint64_t now = tc::global_ns();
       if (it == 255u) t0 = now;
-      if (__any_sync(0xffffffffu, now - t0 > p.wait_ns)) break;
+      if (__any_sync(0xffffffffu, now - t0 > wait_ns)) return false;
     }
   }
-  return spec_vote(&sh.votes, bar, parity);
+}
+__device__ __forceinline__ void spec_arrived(SpecShared &sh, const SpecParams &p, int x) {
+  const uint32_t bar = smem_u32(&sh.bar[x & 1]), parity = (x >> 1) & 1;
+  if (!spec_wait(bar, parity, p.wait_ns)) spec_late(&sh, bar, parity, p.cs, p.status, p.wait_ns);
 }
 
 // A sum over the cluster: warps, then warp 0 over the warps, then the CTAs'
 // values, combined in rank order on every warp (the same bits everywhere).
-// False when the exchange did not arrive.
-__device__ __forceinline__ bool spec_cluster_sum(SpecShared &sh, const SpecParams &p, float v, int x, uint32_t rank,
-                                                 float &sum) {
+__device__ __forceinline__ float spec_cluster_sum(SpecShared &sh, const SpecParams &p, float v, int x, uint32_t rank) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float wv = warp_sum_bcast(v);
   if (lane == 0) sh.red[warp] = wv;
@@ -1319,16 +1355,14 @@ __device__ __forceinline__ bool spec_cluster_sum(SpecShared &sh, const SpecParam
     const float cta = warp_sum_bcast(lane < 16 ? sh.red[lane] : 0.f);
     spec_send(sh, p, make_float4(cta, 0.f, 0.f, 0.f), x, rank);
   }
-  if (!spec_arrived(sh, p, x)) return false;
-  sum = warp_sum_bcast(lane < p.cs ? sh.slot[x & 1][lane].x : 0.f);
-  return true;
+  spec_arrived(sh, p, x);
+  return warp_sum_bcast(lane < p.cs ? sh.slot[x & 1][lane].x : 0.f);
 }
 
 // The rows' maxima and exponential sums over the cluster from each thread's
 // (m_t, s_t, m_d, s_d), s = sum 2^((x - m) k2): (Mt, Zt, Md, Zd). The same
 // three levels as a sum: warps, warp 0 over the warps, the CTAs.
-__device__ __forceinline__ bool spec_cluster_ms(SpecShared &sh, const SpecParams &p, float4 v, int x, uint32_t rank,
-                                                float4 &ms) {
+__device__ __forceinline__ float4 spec_cluster_ms(SpecShared &sh, const SpecParams &p, float4 v, int x, uint32_t rank) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float4 w = ms4_lanes(v, p.k2);
   if (lane == 0) sh.red4[warp] = w;
@@ -1337,9 +1371,8 @@ __device__ __forceinline__ bool spec_cluster_ms(SpecShared &sh, const SpecParams
     const float4 cta = ms4_lanes(lane < 16 ? sh.red4[lane] : make_float4(-INFINITY, 0.f, -INFINITY, 0.f), p.k2);
     spec_send(sh, p, cta, x, rank);
   }
-  if (!spec_arrived(sh, p, x)) return false;
-  ms = ms4_lanes(lane < p.cs ? sh.slot[x & 1][lane] : make_float4(-INFINITY, 0.f, -INFINITY, 0.f), p.k2);
-  return true;
+  spec_arrived(sh, p, x);
+  return ms4_lanes(lane < p.cs ? sh.slot[x & 1][lane] : make_float4(-INFINITY, 0.f, -INFINITY, 0.f), p.k2);
 }
 
 // DREAMS_DATA_* of a sequence's lengths and parent row (0: valid), one warp;
@@ -1623,8 +1656,6 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
   __syncthreads();
   cluster_wait();
   int n = -1, bonus = 0, xc = 0;  // xc: exchanges that have arrived
-  bool dead = false;              // one did not
-  bool sent = false, agreed = false;  // arrived at the cluster's last barrier; past it
   int writer = 0;  // the CTA that draws the bonus and writes the outputs
   if (!bad) {
     int cur = 0;
@@ -1676,10 +1707,7 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
         }
       }
       const float2 m = make_float2(mt.x, md.x);
-      float4 g;
-      dead = !spec_cluster_ms(sh, p, make_float4(m.x, mt.y, m.y, md.y), xc, rank, g);
-      if (dead) break;
-      ++xc;
+      const float4 g = spec_cluster_ms(sh, p, make_float4(m.x, mt.y, m.y, md.y), xc++, rank);
       const float Mt = g.x, Zd = g.w;
       // this thread's factors to the rows' maxima (its exponentials are
       // relative to its own maxima), and their ratio for the passes
@@ -1710,13 +1738,9 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
             acc1 += spec_w(tv.z, dv.z, ct) + spec_w(tv.w, dv.w, ct);
           }
         }
-        float Pn;
-        dead = !spec_cluster_sum(sh, p, at * (acc0 + acc1), xc, rank, Pn);
-        if (dead) break;
-        ++xc;
+        const float Pn = spec_cluster_sum(sh, p, at * (acc0 + acc1), xc++, rank);
         if (Pn > 0.f) c = c2, Pu = Pn;  // a zero sum (r == q) keeps the residual
       }
-      if (dead) break;
       if (next >= 0) {
         ++n;
         cur = next;
@@ -1741,17 +1765,8 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
           const float slice = warp_sum_bcast(lane < 16 ? sh.red[lane] : 0.f);
           spec_send(sh, p, make_float4(slice, 0.f, 0.f, 0.f), xc, rank, true);
         }
-        __syncwarp();
-        cluster_arrive();  // this CTA has had all exchanges but this, which it has sent
-        sent = true;
-        if (!spec_arrived(sh, p, xc)) {
-          // some CTA gave up before, or (all having sent theirs) it only has to land
-          cluster_wait();
-          agreed = true;
-          const uint32_t bar = smem_u32(&sh.bar[xc & 1]);
-          dead = sh.dead || !__syncthreads_and(tc::mbar_wait_cluster(bar, (xc >> 1) & 1, &sh.zero, p.wait_ns));
-          if (dead) break;
-        }
+        const uint32_t bar = smem_u32(&sh.bar[xc & 1]), parity = (xc >> 1) & 1;
+        if (!spec_wait(bar, parity, p.wait_ns)) spec_late_bonus(&sh, bar, parity, p.status, p.wait_ns);
       }
       const float tr = lane < cs ? sh.slot[xc & 1][lane].x : 0.f;
       // their running sum across the lanes, then the crossing slice
@@ -1781,22 +1796,8 @@ __global__ void __launch_bounds__(SPEC_THREADS) spec_walk_kernel(const SpecParam
       break;
     }
   }
-  // Nothing is written before every CTA of the cluster has had all exchanges but
-  // the bonus's and has sent that. A CTA that gave up tells the others (those it
-  // left without its partials give up in turn); all then leave outputs and cache
-  // alone, and end only after the limit once more, when nothing sent to them
-  // can still be under way.
-  if (!sent) {
-    if (dead && tid < cs) st_cluster_one(&sh.dead, uint32_t(tid));
-    __syncwarp();
-    cluster_arrive();
-  }
-  if (!agreed) cluster_wait();
-  if (dead || sh.dead) {
-    if (tid == 0) flag(p.status, DREAMS_DATA_TIMEOUT);
-    tc::mbar_wait_cluster(smem_u32(&sh.bar[xc & 1]), (xc >> 1) & 1, &sh.zero, p.wait_ns);
-    return;
-  }
+  // (From here on every CTA of the cluster has had all exchanges: it has sent the
+  // bonus's. No CTA ends early: it has had every partial that was sent to it.)
   // outputs: path, drafts then the bonus, lengths; the compaction is shared by
   // the cluster's CTAs
   if (warp == 0) {
