@@ -1585,7 +1585,7 @@ __device__ int spec_slice_draw(SpecShared &sh, const float *et, const float *ed,
 // One cluster of p.cs CTAs per sequence (grid.x = B * cs): the walk with its
 // decisions, the bonus draw, the outputs and the KV compaction. A chain of
 // dependent steps, so its latency is what counts: 16 trees of 32-64 nodes at
-// 128256 bf16 entries took 47.8 us a pass, 32.5 with the root's rows loaded
+// 128256 bf16 entries took 47.8 us a pass, 31.9 with the root's rows loaded
 // while the tree is laid out, exponentials from registers, conflict-free slices, warp
 // maxima by one instruction, the outputs written by the CTA that draws, and the
 // first child's rows prefetched.
